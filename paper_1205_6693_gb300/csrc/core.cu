@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
     }
     // --------------------------------------------------------- sub-rounds ---
     int64_t nCur = nF > a.item_cap ? a.item_cap : nF;
-    if (nF > a.item_cap && leader) atomicExch(&ctl->err, TRUSS_ECHECK);
+    if (nF > a.item_cap && leader) raise_error(&ctl->bar, &ctl->err, TRUSS_ECHECK);
     for (;;) {
       unsigned long long *qn = &ctl->qf[ph % 3];
       if (leader) {
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
           dec[q] = false;
           if (w[q] >= 0) {
             if ((uint32_t)w[q] >= (uint32_t)a.n) {
-              atomicExch(&ctl->err, TRUSS_ECHECK);
+              raise_error(&ctl->bar, &ctl->err, TRUSS_ECHECK);
             } else {
               const int sw = __ldcg(&a.stamp[w[q]]);
               dec[q] = sw == 0 || sw > s;  // alive (possibly pushed this sub-round)
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
       if (nN == 0) break;
       { int4 *t = F; F = N; N = t; }
       nCur = nN > a.item_cap ? a.item_cap : nN;
-      if (nN > a.item_cap && leader) atomicExch(&ctl->err, TRUSS_ECHECK);
+      if (nN > a.item_cap && leader) raise_error(&ctl->bar, &ctl->err, TRUSS_ECHECK);
     }
     if (leader) {
       ctl->levels++;

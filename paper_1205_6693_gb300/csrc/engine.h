@@ -168,6 +168,7 @@ struct PeelCfg {
   int block = 512;
   int variant = 0;  // kernel shape (peel.cu: run_peel)
   int sms = 0;
+  int max_sms = 0;  // use at most this many SMs (0 = no limit)
   long long wait_ns = 4000000000LL;
   // Optional: edges never removed (their triangles still count), and the
   // last level to run (0 = all).  Edges not removed by then get truss 0.

@@ -22,37 +22,56 @@
 //
 // Load balance inside a sub-round (its time is that of the slowest warp):
 // an edge that joins a frontier is staged by the warp that pushed it and
-// expanded, when that warp flushes, into work items of kItem list entries
-// each (at least one item, which also records its truss number); an
-// item carries its edge, its entry count and the offset of its entries, so a
-// warp goes from the item straight to the list.  Every warp takes 4 items per
-// iteration, 8 lanes per item and 2 entries per lane (independent loads in
-// flight).  A warp's share of a sub-round is then at most
-// ceil(items / (4 * warps)) iterations, whatever the lengths of the lists.
+// expanded, when that warp flushes, into work items, the aligned 16-entry
+// blocks that its list touches; an item carries its edge, its block number
+// and the part of the block that is the list's, so a warp goes from the item
+// straight to the list.  Every warp takes 4 items per iteration, 8 lanes per
+// item and 2 entries per lane (one 16-byte load).  A warp's share of a
+// sub-round is then at most ceil(items / (4 * warps)) iterations, whatever
+// the lengths of the lists, and the warps that share a small sub-round sit on
+// different SMs.
 // Appends are staged per warp in shared memory and flushed with one atomic
 // reservation per buffer (the list lengths and offsets of a buffer's pushed
-// edges are loaded together at the flush), and per-level reductions (minimum residual, alive
-// count) are combined per block first: a single global counter hit by every
-// warp would serialise the whole grid on one L2 address.
-// Every scan and every sub-round is one phase, ended by one grid barrier.
-// Appends of phase p reserve space through counter slot p % 3 (frontier
-// items qf, alive-list entries qa), which is read after the barrier that
-// ends p.  The leader zeroes slot (p+1) % 3 during phase p: that slot was
-// last read at the start of phase p-1, and every block has passed the
-// barrier ending p-1 before the leader can be in phase p.  A block that
-// leaves a barrier early therefore never appends to a counter that a slow
-// block has still to read.
+// edges are loaded together at the flush, those of an edge whose residual
+// already stood at k-1 together with the decrement that removes it), and
+// per-level reductions (minimum residual, alive count) are combined per block
+// first: a single global counter hit by every warp would serialise the whole
+// grid on one L2 address.
 //
-// Edge state is one 16-bit tag per edge, stamp[e]: 0 = alive, tag(s) = in
-// the frontier of sub-round s, any other value = removed earlier.  A partner
-// pushed during sub-round s is tagged tag(s+1), which reads as alive during
-// s, so one grid barrier per sub-round suffices.  Tags repeat every 65,534
-// sub-rounds, so at least every 32,768 sub-rounds one extra grid-wide pass
-// rewrites every tag but the current frontier's to kDead.  (A 2-byte stamp
-// leaves more of L2 to the residuals, which are read at random.)  res[e] of
-// a frontier edge is never touched during its sub-round and equals the
-// number of its still-alive triangles, so a frontier edge with res 0 skips
-// its list.
+// What bounds it: below about 16 K items a sub-round is a chain of dependent
+// L2 round trips (about 540 clocks each, 900 from HBM): item, list entries,
+// partners' words, decrement, reservation, the release of the barrier's
+// arrival and its polling; above, the random word reads and decrements.  So
+// each step of the chain that can share a load with another does: an edge's
+// state and its residual are one word, the count of a phase's items rides on
+// its barrier's word, and one thread per block reads it.  Sub-rounds of at
+// most 64 items 5.5 -> 4.2 us, scans of short alive lists 8.7 -> 5.0 us; the
+// peel of R-MAT scale 20 27.4 -> 25.6 ms, of a 40 M-edge Chung-Lu graph 77.7
+// -> 72.1 ms, of 4,096 small graphs 10.4 -> 7.6 ms, of the 4,096-vertex graph
+// 0.205 -> 0.131 ms.  Kept in registers, the rarely used state spilled, and
+// every reload after a barrier was one more round trip: it lives in shared
+// memory or is derived.
+// Every scan and every sub-round is one phase, ended by one grid barrier.
+// Appends of phase p reserve space through counter slot p % 3, which is read
+// by the barrier that ends p.  The leader zeroes slot (p+1) % 3 during phase
+// p: that slot was last read at the end of phase p-2, and every block has
+// passed the barrier ending p-1 before the leader can be in phase p.  A block
+// that leaves a barrier early therefore never appends to a counter that a
+// slow block has still to read.
+//
+// Edge state is one 32-bit word per edge: an alive edge's word is its
+// residual (below 2^31); a removed one's has the top bit set, a 16-bit tag
+// and, below it, the residual it was removed with.  tag(s) = in the frontier
+// of sub-round s, any other tag = removed earlier.  An edge whose residual
+// crosses in sub-round s is marked by adding the top bit and tag(s+1) to its
+// word, so that decrements of the same sub-round still land in the residual;
+// marked or not yet, it reads as alive during s, so one grid barrier per
+// sub-round suffices.  Tags repeat every 65,534 sub-rounds, so at least every
+// 32,768 sub-rounds one extra grid-wide pass rewrites every tag but the
+// current frontier's to kDead.  The residual of a frontier edge is never
+// touched during its sub-round and equals the number of its still-alive
+// triangles, so a frontier edge with residual 0 skips its list (one found by
+// the scan is not even queued).
 //
 // Every grid barrier waits at most `wait_ns` (globaltimer); on timeout the
 // kernel records TRUSS_ETIMEOUT and all blocks return at their next barrier.
@@ -73,18 +92,28 @@ constexpr int kItem = 16;  // list entries per work item (8 lanes x 2)
 constexpr int kWP = 32;    // pushed edges staged per warp (one per lane)
 constexpr int kWA = 128;   // alive-list entries staged per warp
 
+// What a scan found (slot = scan index % 3).
+struct __align__(16) ScanOut {
+  int minres;  // least residual of the edges left alive
+  int live;    // how many
+  int any;     // non-zero: the scan removed an edge
+  int listed;  // entries of the rewritten alive list
+};
+
 struct PeelCtl {
-  unsigned long long bar;    // barrier arrivals so far (never reset)
+  // Phase p (slot p % 3): barrier arrivals (bits 0 .. 15), frontier items
+  // appended (16 .. 62); top bit: some block has recorded an error.
+  unsigned long long phase[3];
   int err;
   int pad0;
-  unsigned long long qf[3];  // frontier items appended in phase p (slot p % 3)
-  unsigned long long qa[3];  // alive-list entries appended in phase p
-  int minres[3];             // per scan (slot = scan index % 3)
-  int live[3];               // alive edges left after each scan
+  ScanOut scan[3];
   int levels, subrounds, kmax, ntrace;
   unsigned long long entries, decrements, scanned;
   unsigned long long dead, dead_earlier;  // counting runs
 };
+
+constexpr int kItemShift = 16;
+constexpr unsigned long long kArriveMask = (1ull << kItemShift) - 1;
 
 struct PeelArgs {
   int64_t m;
@@ -95,13 +124,14 @@ struct PeelArgs {
   const int32_t *own_cnt;  // null: no own parts
   const int2 *rest;
   const int64_t *off;
-  int32_t *res;
-  uint16_t *stamp;
-  int retag;  // sub-rounds between tag rewrites (1 .. kRetagMax)
+  uint32_t *word;  // state of each edge (alive: its residual; else kGone | tag | residual)
+  int retag;       // sub-rounds between tag rewrites (1 .. kRetagMax)
   int32_t *truss;
   int32_t *alive0, *alive1;
-  int4 *Q0, *Q1;      // frontier work items (make_item)
-  int64_t item_cap;   // capacity of Q0 and Q1
+  // frontier work items (make_item): one queue grows from the front of Q, the
+  // other from its end; every edge is pushed once, so the two never meet
+  int4 *Q;
+  uint32_t item_cap;  // capacity of Q
   int4 *trace;        // optional: per phase (k, items or -1 for a scan, globaltimer lo/hi)
   int trace_cap;
   PeelCtl *ctl;
@@ -119,79 +149,110 @@ __device__ __forceinline__ void prefetch_l1(const void *p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-__device__ __forceinline__ int items_of(int len) { return len > 0 ? (len + kItem - 1) / kItem : 1; }
-
 constexpr int kTagMod = 65534;
 constexpr int kRetagMax = 32768;
-constexpr uint16_t kDead = 0xFFFF;
+constexpr uint32_t kDead = 0xFFFF;
 // Tag of sub-round s >= 1: 1 .. kTagMod.
-__device__ __forceinline__ uint16_t tag_of(int s) { return (uint16_t)(1 + (s - 1) % kTagMod); }
+__device__ __forceinline__ uint32_t tag_of(int s) { return (uint32_t)(1 + (s - 1) % kTagMod); }
 
-// A work item covers up to kItem consecutive entries of one edge's list:
-// na from its own part at offset oa, then nb from its rest part at ob.
-// Offsets have 42 bits (x = edge, y = na | nb << 5 | first << 10 | the high
-// 10 bits of oa << 11 | those of ob << 21, z / w = the low words of oa / ob).
-constexpr int64_t kOffLimit = (int64_t)1 << 42;
+// A removed edge's word: kGone, its tag in bits 15 .. 30, its residual (at
+// most k - 2, so levels end at kResMax + 2) in the low 15 bits.
+constexpr uint32_t kGone = 0x80000000u;
+constexpr int kTagShift = 15;
+constexpr uint32_t kResMax = (1u << kTagShift) - 1;
+__device__ __forceinline__ uint32_t gone_tag(uint32_t tag) { return kGone | (tag << kTagShift); }
 
-__device__ __forceinline__ int4 make_item(int e, int na, int nb, bool first, int64_t oa,
-                                          int64_t ob) {
-  const uint32_t hi = (uint32_t)na | ((uint32_t)nb << 5) | ((uint32_t)first << 10) |
-                      ((uint32_t)((uint64_t)oa >> 32) & 0x3FFu) << 11 |
-                      ((uint32_t)((uint64_t)ob >> 32) & 0x3FFu) << 21;
-  return make_int4(e, (int)hi, (int)(uint32_t)oa, (int)(uint32_t)ob);
+// A work item is one aligned block of kItem list entries of one edge, the
+// entries [lo, hi) of block `blk` of the own parts or of the rest array: x =
+// edge, y = blk, z = lo | hi << 8 | own << 16 | first << 17 (the item that
+// records the edge's truss number).  Aligned blocks put an item in
+// one 128-byte line and let a lane load its two entries as one 16-byte word.
+constexpr int64_t kOffLimit = (int64_t)kItem << 32;
+
+// Blocks that [off, off + len) touches.
+__device__ __forceinline__ int blocks_of(int64_t off, int len) {
+  return len > 0 ? (int)(((off + len + kItem - 1) >> 4) - (off >> 4)) : 0;
+}
+
+__device__ __forceinline__ int4 make_item(int e, int64_t off, int len, int b, bool own,
+                                          bool first) {
+  const int64_t blk = (off >> 4) + b;
+  const int lo = b == 0 ? (int)(off & (kItem - 1)) : 0;
+  const int64_t left = off + len - (blk << 4);
+  const int hi = left < kItem ? (int)left : kItem;
+  return make_int4(e, (int)(uint32_t)blk, lo | (hi << 8) | ((int)own << 16) | ((int)first << 17),
+                   0);
 }
 
 // Per-warp staging buffers in shared memory (counts are warp-uniform).
 struct WarpBuf {
-  int32_t *push;  // edges pushed to the next frontier, not yet expanded
+  int4 *push;  // pushed edges not yet expanded: edge, list length (-1: not known yet), offset
   int np;
   int32_t *alive;
   int na;
 };
 
+// One of the two item queues: item i is at p[i] (d = 1) or p[-i] (d = -1).
+struct Queue {
+  int4 *Q;
+  uint32_t cap;
+  bool rev;
+  __device__ __forceinline__ int4 *at(uint32_t i) const { return Q + (rev ? cap - 1 - i : i); }
+};
+
+// Reserve n items of phase word *w; the index of the first.
+__device__ __forceinline__ uint32_t reserve_items(unsigned long long *w, int n) {
+  return (uint32_t)(atomicAdd(w, (unsigned long long)(unsigned)n << kItemShift) >> kItemShift);
+}
+
 // Expand the staged pushed edges into work items and append them to queue Q
 // with one reservation.  The list length and offsets of all staged edges
 // are loaded together here, once per flush, instead of one dependent round
 // trip per push inside the sub-round's loop.
-template <bool OWN>
-__device__ __forceinline__ void flush_push(const PeelArgs &a, WarpBuf &wb, int4 *Q,
+__device__ __forceinline__ void flush_push(const PeelArgs &a, WarpBuf &wb, const Queue &Q,
                                            unsigned long long *qctr) {
   const int np = wb.np;
   if (np == 0) return;
   const int lane = lane_id();
   const bool v = lane < np;
-  const int p = v ? wb.push[lane] : 0;
-  const int L = v ? __ldg(&a.sup[p]) : 0;
-  const int64_t lb = v ? __ldg(&a.off[p]) : 0;
-  const int cA = (OWN && v) ? __ldg(&a.own_cnt[p]) : 0;
-  const int64_t la = (OWN && v) ? __ldg(&a.own_off[p]) : 0;
-  const int n = v ? items_of(L) : 0;
+  const int4 st = v ? wb.push[lane] : make_int4(0, 0, 0, 0);
+  const int p = st.x;
+  int L = st.y;
+  int64_t lb = (int64_t)((uint64_t)(uint32_t)st.w << 32 | (uint32_t)st.z);
+  if (L < 0) {
+    L = __ldg(&a.sup[p]);
+    lb = __ldg(&a.off[p]);
+  }
+  const bool own = a.own_cnt != nullptr;
+  const int cA = (own && v) ? __ldg(&a.own_cnt[p]) : 0;
+  const int64_t la = (own && v) ? __ldg(&a.own_off[p]) : 0;
+  L -= cA;  // the rest part
+  const int nA = blocks_of(la, cA);
+  const int n = nA + blocks_of(lb, L);
   const int P = warp_incl_scan(n);
+  uint32_t b = 0;
+  if (lane == 31) b = reserve_items(qctr, P);
   const int tot = __shfl_sync(TR_FULL, P, 31);
-  unsigned long long b = 0;
-  if (lane == 0) b = atomicAdd(qctr, (unsigned long long)tot);
-  const long long base = (long long)__shfl_sync(TR_FULL, b, 0);
+  const uint32_t base = __shfl_sync(TR_FULL, b, 31);
   for (int u0 = 0; u0 < tot; u0 += 32) {
     const int t = u0 + lane;
     const int o = warp_owner(P, t < tot ? t : tot - 1);
     const int po = __shfl_sync(TR_FULL, p, o);
-    const int Po = __shfl_sync(TR_FULL, P, o);
-    const int no = __shfl_sync(TR_FULL, n, o);
+    const int i0 = __shfl_sync(TR_FULL, P - n, o);
     const int Lo = __shfl_sync(TR_FULL, L, o);
-    const int cAo = OWN ? __shfl_sync(TR_FULL, cA, o) : 0;
-    const int64_t lao = OWN ? __shfl_sync(TR_FULL, la, o) : 0;
     const int64_t lbo = __shfl_sync(TR_FULL, lb, o);
-    const long long idx = base + t;
+    int nAo = 0, cAo = 0;
+    int64_t lao = 0;
+    if (own) {
+      nAo = __shfl_sync(TR_FULL, nA, o);
+      cAo = __shfl_sync(TR_FULL, cA, o);
+      lao = __shfl_sync(TR_FULL, la, o);
+    }
+    const uint32_t idx = base + t;
     if (t < tot && idx < a.item_cap) {
-      const int it = t - (Po - no);
-      const int start = it * kItem;
-      const int cnt = Lo > 0 ? min(kItem, Lo - start) : 0;
-      const int na = min(max(cAo - start, 0), cnt);
-      Q[idx] = make_item(po, na, cnt - na, it == 0, lao + start, lbo + max(start - cAo, 0));
+      const int it = t - i0;
+      *Q.at(idx) = it < nAo ? make_item(po, lao, cAo, it, true, it == 0)
+                            : make_item(po, lbo, Lo, it - nAo, false, it == 0);
     }
   }
   __syncwarp();
@@ -199,12 +260,12 @@ __device__ __forceinline__ void flush_push(const PeelArgs &a, WarpBuf &wb, int4 
 }
 
 __device__ __forceinline__ void flush_alive(const PeelArgs &a, WarpBuf &wb, int32_t *A2,
-                                            unsigned long long *actr) {
+                                            int *actr) {
   if (wb.na == 0) return;
   const int lane = lane_id();
-  unsigned long long b = 0;
-  if (lane == 0) b = atomicAdd(actr, (unsigned long long)wb.na);
-  const long long b0 = (long long)__shfl_sync(TR_FULL, b, 0);
+  int b = 0;
+  if (lane == 0) b = atomicAdd(actr, wb.na);
+  const int b0 = __shfl_sync(TR_FULL, b, 0);
   for (int t = lane; t < wb.na; t += 32)
     if (b0 + t < a.m) A2[b0 + t] = wb.alive[t];
   __syncwarp();
@@ -213,7 +274,7 @@ __device__ __forceinline__ void flush_alive(const PeelArgs &a, WarpBuf &wb, int3
 
 // Queue the alive edges of the lanes with `keep` for the rewritten list.
 __device__ __forceinline__ void push_alive(const PeelArgs &a, bool keep, int e, WarpBuf &wb,
-                                           int32_t *A2, unsigned long long *actr) {
+                                           int32_t *A2, int *actr) {
   const unsigned mask = __ballot_sync(TR_FULL, keep);
   if (mask == 0) return;
   const int tot = __popc(mask);
@@ -223,158 +284,120 @@ __device__ __forceinline__ void push_alive(const PeelArgs &a, bool keep, int e, 
   wb.na += tot;
 }
 
-// Push edge p (for each lane with `push`) to the next frontier: stamp it
-// with tag `tagv` and stage it for expansion into work items.  All lanes
-// call it.
-template <bool OWN>
-__device__ __forceinline__ void push_items(const PeelArgs &a, bool push, int p, WarpBuf &wb,
-                                           int4 *Q, unsigned long long *qctr, uint16_t tagv) {
+__device__ __forceinline__ void prefetch_list(const PeelArgs &a, int p) {
+  prefetch_l1(a.sup + p);
+  prefetch_l1(a.off + p);
+  if (a.own_cnt) {
+    prefetch_l1(a.own_cnt + p);
+    prefetch_l1(a.own_off + p);
+  }
+}
+
+// Stage edge p (for each lane with `push`) for expansion into work items of
+// the next frontier.  All lanes call it.
+__device__ __forceinline__ void push_items(const PeelArgs &a, bool push, int4 p, WarpBuf &wb,
+                                           const Queue &Q, unsigned long long *qctr) {
   const unsigned mask = __ballot_sync(TR_FULL, push);
   if (mask == 0) return;
   const int tot = __popc(mask);
-  if (wb.np + tot > kWP) flush_push<OWN>(a, wb, Q, qctr);
+  if (wb.np + tot > kWP) flush_push(a, wb, Q, qctr);
   if (push) {
-    a.stamp[p] = tagv;
     wb.push[wb.np + __popc(mask & ((1u << lane_id()) - 1u))] = p;
-    // the flush reads p's list length and offsets: start fetching them now
-    prefetch_l1(a.sup + p);
-    prefetch_l1(a.off + p);
-    if (OWN) {
-      prefetch_l1(a.own_cnt + p);
-      prefetch_l1(a.own_off + p);
-    }
+    if (p.y < 0) prefetch_list(a, p.x);  // the flush reads its list length and offsets
   }
   __syncwarp();
   wb.np += tot;
 }
 
-// Decide whether frontier edge e charges the triangle {e, p1, p2} in
-// sub-round s: all three edges alive, and e the lowest-id frontier edge among
-// them.  d1 / d2 = decrement p1 / p2 (the partners not in the frontier).
-// ts / tn = tag(s) / tag(s+1).
-__device__ __forceinline__ void decide(const PeelArgs &a, bool valid, int e, int2 pr, int ts,
-                                       int tn, bool &d1, bool &d2, bool &dead) {
-  d1 = d2 = dead = false;
-  if (!valid) return;
-  const int p1 = pr.x, p2 = pr.y;
-  if ((uint32_t)p1 >= (uint32_t)a.m || (uint32_t)p2 >= (uint32_t)a.m) {
-    atomicExch(&a.ctl->err, TRUSS_ECHECK);  // corrupt list entry: skip it
-    return;
-  }
-  // more than half the entries read belong to triangles that already lost
-  // an edge: partner 2's state is read only if partner 1 is still there
-  const int s1 = __ldcg(&a.stamp[p1]);
-  if (s1 != 0 && s1 != ts && s1 != tn) {
-    dead = true;
-    return;
-  }
-  const int s2 = __ldcg(&a.stamp[p2]);
-  const bool dead1 = s1 != 0 && s1 != ts && s1 != tn, dead2 = s2 != 0 && s2 != ts && s2 != tn;
-  dead = dead1 || dead2;
-  if (dead) return;
-  const bool in1 = s1 == ts, in2 = s2 == ts;
-  if (!in1 && !in2) {
-    d1 = true;
-    d2 = true;
-  } else if (in1 && !in2) {
-    d2 = e < p1;  // e and e1 in F: the lower id charges e2
-  } else if (!in1 && in2) {
-    d1 = e < p2;
-  }
+// What a partner's word says in the sub-round whose frontier carries word
+// prefix fs (gone_tag(tag(s)) >> kTagShift) and whose pushes carry fn.
+__device__ __forceinline__ bool in_front(uint32_t w, uint32_t fs) { return (w >> kTagShift) == fs; }
+__device__ __forceinline__ bool is_dead(uint32_t w, uint32_t fs, uint32_t fn) {
+  const uint32_t h = w >> kTagShift;
+  return (int32_t)w < 0 && h != fs && h != fn;
 }
 
-// NE triangle entries per lane (all lanes call it; `v[i]` masks idle
-// entries, e[i] is the frontier edge of entry i).  Each charged triangle
-// decrements its partners outside the frontier; a partner whose residual
-// crosses k-1 -> k-2 joins the next frontier.  All loads and atomics of the
-// NE entries are issued before any result is used.
-template <int NE, bool OWN, bool COUNT>
-__device__ __forceinline__ void charge(const PeelArgs &a, const int *e, const bool *v,
-                                       const int2 *p, int k, int ts, int tn, WarpBuf &wb,
-                                       int4 *N, unsigned long long *qctr,
-                                       unsigned &n_dec, int s_lvl0, unsigned &n_dead,
-                                       unsigned &n_early) {
-  bool d1[NE], d2[NE], dd[NE];
-#pragma unroll
-  for (int i = 0; i < NE; i++) decide(a, v[i], e[i], p[i], ts, tn, d1[i], d2[i], dd[i]);
-  if (COUNT) {
-    // a destroyed triangle lost its first edge when the earlier-removed of
-    // its removed partners went (partners still alive have no removal yet)
-#pragma unroll
-    for (int i = 0; i < NE; i++) {
-      if (!dd[i]) continue;
-      const int w1 = __ldcg(&a.when[p[i].x]), w2 = __ldcg(&a.when[p[i].y]);
-      n_dead++;
-      n_early += min(w1, w2) < s_lvl0;
+// End of a phase: a barrier of the whole grid, after which *items is the number of items the phase appended and, for a
+// scan, *so is what it found.  The count shares its word with the barrier's
+// arrivals, so the load that sees the last arrival brings it along, and one
+// thread per block reads and passes it on: read by every warp, one L2 sector
+// served 4,864 requests per value and barrier (1.1 us of each sub-round, 5
+// to 7 us of each scan).  A grid barrier that waits longer than wait_ns
+// records TRUSS_ETIMEOUT.  Returns false if some block has recorded an error.
+__device__ __forceinline__ bool phase_end(const PeelArgs &a, unsigned ph, uint32_t *items,
+                                          const ScanOut *scan, ScanOut *so) {
+  __shared__ unsigned long long s_word2[2];  // by phase parity: read until the next phase ends
+  __shared__ ScanOut s_scan2[2];
+  unsigned long long &s_word = s_word2[ph & 1];
+  ScanOut &s_scan = s_scan2[ph & 1];
+  unsigned long long *w = &a.ctl->phase[ph % 3];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long v = atom_add_acq_rel_gpu(w, 1ull) + 1;
+    if ((v & kArriveMask) != gridDim.x) {
+      const unsigned long long t0 = global_ns();
+      for (unsigned spins = 1;; spins++) {
+        v = ld_acquire_gpu(w);
+        if ((v & kArriveMask) == gridDim.x || (v & kBarErr)) break;
+        if (spins > 32) __nanosleep(32);
+        if ((spins & 15) == 0 && (long long)(global_ns() - t0) > a.wait_ns) {
+          raise_error(w, &a.ctl->err, TRUSS_ETIMEOUT);
+          v = kBarErr;
+          break;
+        }
+      }
     }
+    s_word = v;
+    if (scan) *(int4 *)&s_scan = __ldcg((const int4 *)scan);
   }
-  int o1[NE], o2[NE];
-#pragma unroll
-  for (int i = 0; i < NE; i++) {
-    o1[i] = d1[i] ? atomicSub(&a.res[p[i].x], 1) : INT_MAX;
-    o2[i] = d2[i] ? atomicSub(&a.res[p[i].y], 1) : INT_MAX;
-    n_dec += (unsigned)(d1[i] + d2[i]);
-  }
-  // pending pushes of this lane, bit 2i (p[i].x) and 2i+1 (p[i].y); the
-  // warp pushes one per lane per step through a single push_items site
-  unsigned pend = 0;
-#pragma unroll
-  for (int i = 0; i < NE; i++)
-    pend |= (o1[i] == k - 1 ? 1u : 0u) << (2 * i) | (o2[i] == k - 1 ? 1u : 0u) << (2 * i + 1);
-  while (__any_sync(TR_FULL, pend != 0)) {
-    int q = 0;
-    const bool has = pend != 0;
-    if (has) {
-      const int b = __ffs(pend) - 1;
-      pend &= pend - 1;
-#pragma unroll
-      for (int i = 0; i < NE; i++)
-        if ((b >> 1) == i) q = (b & 1) ? p[i].y : p[i].x;
-    }
-    push_items<OWN>(a, has, q, wb, N, qctr, (uint16_t)tn);
-  }
+  __syncthreads();
+  const unsigned long long v = s_word;
+  *items = (uint32_t)((v & ~kBarErr) >> kItemShift);
+  if (scan) *so = s_scan;
+  return (v & kBarErr) == 0;
 }
 
 // MINB = resident blocks per SM the register budget is sized for (1: up to
 // 128 registers per thread, 2: 64); G = work items per 8-lane group per
 // iteration (2 entries per lane per item).
-// OWN: the lists keep own parts in the records (TriLists::own_cnt set).
-template <int MINB, int G, bool OWN, bool COUNT = false>
+template <int MINB, int G, bool COUNT = false>
 __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
   const int lane = lane_id();
   const int wib = threadIdx.x >> 5;
-  const int gwarp = blockIdx.x * kWarps + wib;  // grids are one or two blocks per SM
+  // consecutive warps of the launch sit in different blocks, so a phase with
+  // little work spreads it over all SMs
+  const int gwarp = wib * gridDim.x + blockIdx.x;
   const int twarps = gridDim.x * kWarps;
   const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
   PeelCtl *ctl = a.ctl;
-  __shared__ int32_t s_push[kWarps][kWP];
+  __shared__ int4 s_push[kWarps][kWP];
   __shared__ int32_t s_alive[kWarps][kWA];
-  __shared__ int s_minres, s_live;
+  __shared__ int s_minres, s_live, s_any;
   WarpBuf wb{s_push[wib], 0, s_alive[wib], 0};
   if (threadIdx.x == 0) {
     s_minres = INT_MAX;
     s_live = 0;
+    s_any = 0;
   }
   __syncthreads();
 
   int k = 2, s = 1, sc = 0;
   unsigned ph = 0;  // phase index (scans and sub-rounds)
-  int32_t *alive = a.alive0, *alive2 = a.alive1;
-  int4 *F = a.Q0, *N = a.Q1;
-  int64_t nAlive = a.m;
+  bool odd = false;  // which alive list is current
+  bool rev = false;  // which queue is the current frontier's
+  int nAlive = (int)a.m;
   bool compact = false;  // rewrite the alive list during this scan
-  // per-lane work counts (32-bit: a lane's share of even 2^33 list entries
-  // over the grid's 150 K lanes stays far below 2^32)
-  unsigned n_entries = 0, n_dec = 0, n_scan = 0;
+  // work counts of each thread, in shared memory: registers are short (32-bit:
+  // a lane's share of even 2^33 list entries over the grid's 150 K lanes stays
+  // far below 2^32)
+  __shared__ uint2 s_work[kPeelBlock];  // entries read, decrements
+  s_work[threadIdx.x] = make_uint2(0, 0);
   unsigned n_dead = 0, n_early = 0;  // counting runs: totals so far
-  // this warp's first work items of the coming sub-round, loaded right after
-  // the barrier together with the item count instead of after it
-  int4 pre[G];
-  const int64_t it0 = (int64_t)gwarp * 4 * G + (lane >> 3);
-  auto prefetch = [&](const int4 *Q) {
-#pragma unroll
-    for (int g = 0; g < G; g++)
-      pre[g] = it0 + g * 4 < a.item_cap ? __ldcg(&Q[it0 + g * 4]) : make_int4(0, 0, 0, 0);
+  auto clamp = [&](uint32_t n) {
+    if (n <= a.item_cap) return n;
+    // appends beyond the queue were dropped
+    if (leader) raise_error(&ctl->phase[ph % 3], &ctl->err, TRUSS_ECHECK);
+    return a.item_cap;
   };
   // Every a.retag sub-rounds (checked at the start of each phase, the same in
   // every block): tags other than the current frontier's become kDead.  A
@@ -384,59 +407,80 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
   auto retag = [&]() -> bool {
     if (s - last_retag < a.retag) return true;
     last_retag = s;
-    const uint16_t keep = tag_of(s);
+    if (leader) ctl->phase[(ph + 1) % 3] = 0;
+    const uint32_t keep = gone_tag(tag_of(s)) >> kTagShift;
     const int64_t nt = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < a.m; e += nt) {
-      const uint16_t t = __ldcg(&a.stamp[e]);
-      if (t != 0 && t != keep) a.stamp[e] = kDead;
+      const uint32_t w = __ldcg(&a.word[e]);
+      if ((int32_t)w < 0 && (w >> kTagShift) != keep)
+        a.word[e] = gone_tag(kDead) | (w & kResMax);
     }
-    return grid_barrier(&ctl->bar, &ctl->err, a.wait_ns);
+    uint32_t items;
+    const bool ok = phase_end(a, ph, &items, nullptr, nullptr);
+    ph++;
+    return ok;
   };
 
   for (;;) {
     if (a.k_stop > 0 && k > a.k_stop) break;  // k is the same in every block
+    if (k - 2 > (int)kResMax) {
+      // no graph whose lists fit the device has a truss this deep
+      if (leader) raise_error(&ctl->phase[ph % 3], &ctl->err, TRUSS_ECHECK);
+      break;
+    }
     if (!retag()) return;
     // ------------------------------------------------------------ scan ---
     if (leader && a.trace && ctl->ntrace < a.trace_cap) {
       const unsigned long long t = global_ns();
       a.trace[ctl->ntrace++] = make_int4(k, -1, (int)(uint32_t)t, (int)(uint32_t)(t >> 32));
     }
-    const int slot = sc % 3;
-    unsigned long long *qf = &ctl->qf[ph % 3], *qa = &ctl->qa[ph % 3];
+    ScanOut *scan = &ctl->scan[sc % 3];
+    unsigned long long *qf = &ctl->phase[ph % 3];
     if (leader) {
-      ctl->minres[(sc + 1) % 3] = INT_MAX;
-      ctl->live[(sc + 1) % 3] = 0;
-      ctl->qf[(ph + 1) % 3] = 0;
-      ctl->qa[(ph + 1) % 3] = 0;
+      *(int4 *)&ctl->scan[(sc + 1) % 3] = make_int4(INT_MAX, 0, 0, 0);
+      ctl->phase[(ph + 1) % 3] = 0;
     }
-    int wmin = INT_MAX, wlive = 0;
+    const int32_t *alive = odd ? a.alive1 : a.alive0;
+    int32_t *alive2 = odd ? a.alive0 : a.alive1;
+    const Queue F{a.Q, a.item_cap, rev};
+    int lmin = INT_MAX, llive = 0;  // of this lane
+    bool lany = false;
     // 4 x 32 entries per warp iteration: all loads are issued before any
     // decision, so one dependent round trip covers 4 entries per lane
     constexpr int kScanU = 4;
     for (int64_t base = (int64_t)gwarp * 32 * kScanU; base < nAlive;
          base += (int64_t)twarps * 32 * kScanU) {
-      int e[kScanU], st[kScanU], r[kScanU];
+      int e[kScanU];
+      uint32_t w[kScanU];
 #pragma unroll
       for (int u = 0; u < kScanU; u++) {
         const int64_t i = base + u * 32 + lane;
         e[u] = i < nAlive ? __ldcg(&alive[i]) : -1;
       }
 #pragma unroll
-      for (int u = 0; u < kScanU; u++) {
-        st[u] = e[u] >= 0 ? __ldcg(&a.stamp[e[u]]) : 1;
-        r[u] = e[u] >= 0 ? __ldcg(&a.res[e[u]]) : 0;
-      }
+      for (int u = 0; u < kScanU; u++) w[u] = e[u] >= 0 ? __ldcg(&a.word[e[u]]) : kGone;
       unsigned pend = 0;  // entries of this lane that join the frontier
 #pragma unroll
       for (int u = 0; u < kScanU; u++) {
-        const bool live = e[u] >= 0 && st[u] == 0;
-        const bool toF = live && r[u] <= k - 2;
+        const bool live = (int32_t)w[u] >= 0;
+        const bool toF = live && (int)w[u] <= k - 2;
         const bool keep = live && !toF;
-        pend |= (toF ? 1u : 0u) << u;
-        if (compact) push_alive(a, keep, e[u], wb, alive2, qa);
-        wmin = min(wmin, __reduce_min_sync(TR_FULL, keep ? r[u] : INT_MAX));
-        wlive += __popc(__ballot_sync(TR_FULL, keep));
-        n_scan += (e[u] >= 0);
+        if (toF) {
+          // removed at this level; without triangles left it needs no item
+          a.word[e[u]] = gone_tag(tag_of(s)) | w[u];
+          if (w[u] > 0) {
+            pend |= 1u << u;
+          } else {
+            a.truss[e[u]] = k;
+            if (COUNT) a.when[e[u]] = s;
+          }
+          lany = true;
+        }
+        if (compact) push_alive(a, keep, e[u], wb, alive2, &scan->listed);
+        if (keep) {
+          lmin = min(lmin, (int)w[u]);
+          llive++;
+        }
       }
       while (__any_sync(TR_FULL, pend != 0)) {
         int q = 0;
@@ -448,141 +492,219 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
           for (int u = 0; u < kScanU; u++)
             if (b == u) q = e[u];
         }
-        push_items<OWN>(a, has, q, wb, F, qf, tag_of(s));
+        push_items(a, has, make_int4(q, -1, 0, 0), wb, F, qf);
       }
     }
-    flush_push<OWN>(a, wb, F, qf);
-    if (compact) flush_alive(a, wb, alive2, qa);
-    if (lane == 0) {
-      if (wmin != INT_MAX) atomicMin(&s_minres, wmin);
-      if (wlive) atomicAdd(&s_live, wlive);
+    flush_push(a, wb, F, qf);
+    if (compact) flush_alive(a, wb, alive2, &scan->listed);
+    if ((int64_t)gwarp * 32 * kScanU < nAlive) {
+      lmin = __reduce_min_sync(TR_FULL, lmin);
+      llive = __reduce_add_sync(TR_FULL, llive);
+      const bool wany = __any_sync(TR_FULL, lany);
+      if (lane == 0) {
+        if (lmin != INT_MAX) atomicMin(&s_minres, lmin);
+        if (llive) atomicAdd(&s_live, llive);
+        if (wany) s_any = 1;
+      }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      if (s_minres != INT_MAX) atomicMin(&ctl->minres[slot], s_minres);
-      if (s_live) atomicAdd(&ctl->live[slot], s_live);
+      if (s_minres != INT_MAX) atomicMin(&scan->minres, s_minres);
+      if (s_live) atomicAdd(&scan->live, s_live);
+      if (s_any) scan->any = 1;
       s_minres = INT_MAX;
       s_live = 0;
+      s_any = 0;
     }
-    if (!grid_barrier(&ctl->bar, &ctl->err, a.wait_ns)) return;
+    uint32_t nCur;  // items of the frontier
+    ScanOut found;
+    if (!phase_end(a, ph, &nCur, scan, &found)) return;
     ph++;
-    prefetch(F);
-    const int minres = __ldcg(&ctl->minres[slot]);
-    const int64_t live = __ldcg(&ctl->live[slot]);
-    const int64_t nF = (int64_t)__ldcg(qf);
+    const int minres = found.minres, live = found.live, any = found.any;
+    if (leader) ctl->scanned += (unsigned)nAlive;
     if (compact) {
-      nAlive = (int64_t)__ldcg(qa);
-      int32_t *t = alive;
-      alive = alive2;
-      alive2 = t;
+      nAlive = found.listed;
+      odd = !odd;
     }
-    compact = 4 * live <= 3 * nAlive;  // rewrite the list once a quarter of it is dead
+    compact = 4 * (int64_t)live <= 3 * (int64_t)nAlive;  // rewrite the list once a quarter of it is dead
     sc++;
-    if (nF == 0) {
+    if (any && leader) {
+      ctl->levels++;
+      ctl->kmax = k;
+    }
+    if (nCur == 0) {
+      // nothing removed had a triangle left, so the residuals stand
       if (live == 0) break;
       k = minres + 2;  // every alive edge has res >= k-1: skip empty levels
       continue;
     }
     // --------------------------------------------------------- sub-rounds ---
-    int64_t nCur = nF;
+    nCur = clamp(nCur);
     const int s_lvl0 = s;  // first sub-round of this level
     for (;;) {
-      const unsigned c_ent = n_entries, c_dead = n_dead, c_early = n_early;
+      const unsigned c_ent = COUNT ? s_work[threadIdx.x].x : 0, c_dead = n_dead, c_early = n_early;
       if (!retag()) return;
-      const int ts = tag_of(s), tn = tag_of(s + 1);
+      const uint32_t fs = gone_tag(tag_of(s)) >> kTagShift, pushw = gone_tag(tag_of(s + 1)),
+                     fn = pushw >> kTagShift;
       if (leader && a.trace && ctl->ntrace < a.trace_cap) {
         const unsigned long long t = global_ns();
-        a.trace[ctl->ntrace++] = make_int4(k, (int)min(nCur, (int64_t)INT_MAX),
+        a.trace[ctl->ntrace++] = make_int4(k, (int)min(nCur, (uint32_t)INT_MAX),
                                            (int)(uint32_t)t, (int)(uint32_t)(t >> 32));
       }
-      unsigned long long *qn = &ctl->qf[ph % 3];
-      if (leader) {
-        ctl->qf[(ph + 1) % 3] = 0;
-        ctl->qa[(ph + 1) % 3] = 0;
-      }
+      unsigned long long *qn = &ctl->phase[ph % 3];
+      if (leader) ctl->phase[(ph + 1) % 3] = 0;
       const int grp = lane >> 3, j = lane & 7;
-      const int64_t stride = (int64_t)twarps * 4 * G;
-      for (int64_t base = (int64_t)gwarp * 4 * G; base < nCur; base += stride) {
-        // this iteration's items were loaded one iteration ahead (the first
-        // right after the barrier); load the next iteration's now
-        int4 cur[G];
+      const uint32_t stride = (uint32_t)twarps * 4 * G;
+      const Queue F{a.Q, a.item_cap, rev}, N{a.Q, a.item_cap, !rev};
+      // Items are loaded two iterations ahead and their list entries and
+      // edge words one ahead, so that an iteration waits only for its
+      // partners' words and decrements.
+      int4 cur[G], nxt[G], ent[G], entn[G];  // ent: two list entries of this lane per item
+      uint32_t we[G], wen[G];
+      auto load_item = [&](int4 *it, uint32_t base) {
+#pragma unroll
+        for (int g = 0; g < G; g++)
+          it[g] = base + g * 4 + grp < nCur ? __ldcg(F.at(base + g * 4 + grp))
+                                            : make_int4(0, 0, 0, 0);
+      };
+      auto load_entries = [&](const int4 *it, int4 *en, uint32_t *w) {
 #pragma unroll
         for (int g = 0; g < G; g++) {
-          cur[g] = pre[g];
-          const int64_t nx = base + stride + g * 4 + grp;
-          pre[g] = nx < nCur ? __ldcg(&F[nx]) : make_int4(0, 0, 0, 0);
+          const int lo = it[g].z & 0xFF, hi = (it[g].z >> 8) & 0xFF;
+          const bool any2 = 2 * j + 1 >= lo && 2 * j < hi;
+          w[g] = any2 ? __ldcg(&a.word[it[g].x]) : 0u;
+          // list entries are read once: evict-first, so that the words
+          // (re-read at random) keep their place in L2
+          const int4 *blk = (const int4 *)(((it[g].z >> 16) & 1) ? a.own : a.rest) +
+                            (int64_t)(uint32_t)it[g].y * 8;
+          en[g] = any2 ? __ldcs(blk + j) : make_int4(0, 0, 0, 0);
         }
-        int ee[2 * G];
-        bool vv[2 * G];
-        int2 pp[2 * G];
-        int na[G], cnt[G];
-        int64_t la[G], lb[G];
+      };
+      uint32_t base = (uint32_t)gwarp * 4 * G;
+      if (base < nCur) {
+        load_item(cur, base);
+        load_item(nxt, base + stride);
+        load_entries(cur, ent, we);
+      }
+      for (; base < nCur; base += stride) {
+        load_entries(nxt, entn, wen);
+        int4 nxt2[G];
+        load_item(nxt2, base + 2 * stride);
+        bool v0[G], v1[G];
 #pragma unroll
         for (int g = 0; g < G; g++) {
-          const int64_t it = base + g * 4 + grp;
-          ee[2 * g] = 0;
-          na[g] = 0;
-          cnt[g] = 0;
-          la[g] = 0;
-          lb[g] = 0;
-          if (it < nCur) {
-            const int4 item = cur[g];
-            const uint32_t hi = (uint32_t)item.y;
-            ee[2 * g] = item.x;
-            na[g] = OWN ? (int)(hi & 31u) : 0;
-            cnt[g] = na[g] + ((hi >> 5) & 31u);
-            la[g] = OWN ? (int64_t)(((uint64_t)((hi >> 11) & 0x3FFu) << 32) | (uint32_t)item.z) : 0;
-            lb[g] = (int64_t)(((uint64_t)(hi >> 21) << 32) | (uint32_t)item.w);
-            if (((hi >> 10) & 1u) && j == 0) {
-              a.truss[item.x] = k;
-              if (COUNT) a.when[item.x] = s;
+          const int lo = cur[g].z & 0xFF, hi = (cur[g].z >> 8) & 0xFF;
+          if ((cur[g].z >> 17) && j == 0) {
+            a.truss[cur[g].x] = k;
+            if (COUNT) a.when[cur[g].x] = s;
+          }
+          v0[g] = 2 * j >= lo && 2 * j < hi;
+          v1[g] = 2 * j + 1 >= lo && 2 * j + 1 < hi;
+        }
+        // Charge: a triangle of frontier edge e and partners p1, p2, none
+        // of them removed earlier, is charged by the lowest-id frontier edge
+        // among the three, which decrements the partners not in the frontier.
+        uint2 work = make_uint2(0, 0);
+        uint32_t s1[2 * G], s2[2 * G];
+        bool d1[2 * G], d2[2 * G];
+#pragma unroll
+        for (int i = 0; i < 2 * G; i++) {
+          const int g = i >> 1;
+          const int p1 = (i & 1) ? ent[g].z : ent[g].x, p2 = (i & 1) ? ent[g].w : ent[g].y;
+          bool v = ((i & 1) ? v1[g] : v0[g]) && (we[g] & kResMax) != 0;
+          if (v && ((uint32_t)p1 >= (uint32_t)a.m || (uint32_t)p2 >= (uint32_t)a.m)) {
+            raise_error(&ctl->phase[ph % 3], &ctl->err, TRUSS_ECHECK);  // corrupt list entry: skip it
+            v = false;
+          }
+          work.x += v;
+          // a masked entry reads as dead
+          s1[i] = v ? __ldcg(&a.word[p1]) : gone_tag(0);
+          s2[i] = v ? __ldcg(&a.word[p2]) : gone_tag(0);
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * G; i++) {
+          const int g = i >> 1, e = cur[g].x;
+          const int p1 = (i & 1) ? ent[g].z : ent[g].x, p2 = (i & 1) ? ent[g].w : ent[g].y;
+          const bool dead = is_dead(s1[i], fs, fn) || is_dead(s2[i], fs, fn);
+          const bool in1 = in_front(s1[i], fs), in2 = in_front(s2[i], fs);
+          d1[i] = !dead && !in1 && (!in2 || e < p2);
+          d2[i] = !dead && !in2 && (!in1 || e < p1);
+          if (COUNT) {
+            // a destroyed triangle lost its first edge when the earlier-
+            // removed of its removed partners went
+            const bool v = ((i & 1) ? v1[g] : v0[g]) && (we[g] & kResMax) != 0;
+            if (v && dead && (uint32_t)p1 < (uint32_t)a.m && (uint32_t)p2 < (uint32_t)a.m) {
+              const int w1 = __ldcg(&a.when[p1]), w2 = __ldcg(&a.when[p2]);
+              n_dead++;
+              n_early += min(w1, w2) < s_lvl0;
             }
           }
-          ee[2 * g + 1] = ee[2 * g];
         }
-        int r[G];
+        // a partner that a decrement should remove: fetch its list's place now
+        int cand = -1, candL = 0;
+        int64_t candO = 0;
+#pragma unroll
+        for (int i = 0; i < 2 * G; i++) {
+          const int g = i >> 1;
+          const int p1 = (i & 1) ? ent[g].z : ent[g].x, p2 = (i & 1) ? ent[g].w : ent[g].y;
+          if (d1[i] && s1[i] == (uint32_t)(k - 1)) cand = p1;
+          if (d2[i] && s2[i] == (uint32_t)(k - 1)) cand = p2;
+        }
+        if (cand >= 0) {
+          candL = __ldg(&a.sup[cand]);
+          candO = __ldg(&a.off[cand]);
+        }
+        unsigned pend = 0;  // pending pushes, bit 2i (p1) and 2i+1 (p2)
+#pragma unroll
+        for (int i = 0; i < 2 * G; i++) {
+          const int g = i >> 1;
+          const int p1 = (i & 1) ? ent[g].z : ent[g].x, p2 = (i & 1) ? ent[g].w : ent[g].y;
+          // s1 / s2 take the residuals before the decrements
+          s1[i] = d1[i] ? atomicSub(&a.word[p1], 1u) : 0u;
+          s2[i] = d2[i] ? atomicSub(&a.word[p2], 1u) : 0u;
+          work.y += (unsigned)(d1[i] + d2[i]);
+        }
+        s_work[threadIdx.x].x += work.x;
+        s_work[threadIdx.x].y += work.y;
+#pragma unroll
+        for (int i = 0; i < 2 * G; i++) {
+          // k >= 3 here, so a lane without a decrement (0) never matches
+          pend |= (s1[i] == (uint32_t)(k - 1) ? 1u : 0u) << (2 * i) |
+                  (s2[i] == (uint32_t)(k - 1) ? 1u : 0u) << (2 * i + 1);
+        }
+        // the warp pushes one partner per lane per step through one site
+        while (__any_sync(TR_FULL, pend != 0)) {
+          int q = 0;
+          const bool has = pend != 0;
+          if (has) {
+            const int b = __ffs(pend) - 1;
+            pend &= pend - 1;
+#pragma unroll
+            for (int i = 0; i < 2 * G; i++) {
+              const int g = i >> 1;
+              if ((b >> 1) == i)
+                q = (b & 1) ? ((i & 1) ? ent[g].w : ent[g].y) : ((i & 1) ? ent[g].z : ent[g].x);
+            }
+            // others may still decrement q's residual: add the mark to it
+            atomicAdd(&a.word[q], pushw);
+          }
+          const bool known = q == cand;
+          push_items(a, has,
+                     make_int4(q, known ? candL : -1, (int)(uint32_t)candO,
+                               (int)(uint32_t)((uint64_t)candO >> 32)),
+                     wb, N, qn);
+        }
 #pragma unroll
         for (int g = 0; g < G; g++) {
-          const bool ha = j < cnt[g], hb = j + 8 < cnt[g];
-          r[g] = ha ? __ldcg(&a.res[ee[2 * g]]) : 0;
-          // list entries are read once: evict-first, so that the residuals
-          // and stamps (re-read at random) keep their place in L2
-          const int2 *srcA = j < na[g] ? a.own + la[g] + j : a.rest + lb[g] + (j - na[g]);
-          const int2 *srcB =
-              j + 8 < na[g] ? a.own + la[g] + j + 8 : a.rest + lb[g] + (j + 8 - na[g]);
-          pp[2 * g] = ha ? __ldcs(srcA) : make_int2(0, 0);
-          pp[2 * g + 1] = hb ? __ldcs(srcB) : make_int2(0, 0);
-          vv[2 * g] = ha;
-          vv[2 * g + 1] = hb;
+          cur[g] = nxt[g];
+          nxt[g] = nxt2[g];
+          ent[g] = entn[g];
+          we[g] = wen[g];
         }
-#pragma unroll
-        for (int g = 0; g < G; g++) {
-          vv[2 * g] = vv[2 * g] && r[g] > 0;
-          vv[2 * g + 1] = vv[2 * g + 1] && r[g] > 0;
-          n_entries += (unsigned)(vv[2 * g] + vv[2 * g + 1]);
-        }
-        // the next iteration's items have arrived by now: start fetching
-        // their list entries (into L1; the lists are read-only here) and
-        // their edges' residuals (into L2) while this iteration charges
-#pragma unroll
-        for (int g = 0; g < G; g++) {
-          const uint32_t hi = (uint32_t)pre[g].y;
-          const int nna = OWN ? (int)(hi & 31u) : 0;
-          const int ncnt = nna + (int)((hi >> 5) & 31u);
-          const int64_t nla =
-              OWN ? (int64_t)(((uint64_t)((hi >> 11) & 0x3FFu) << 32) | (uint32_t)pre[g].z) : 0;
-          const int64_t nlb = (int64_t)(((uint64_t)(hi >> 21) << 32) | (uint32_t)pre[g].w);
-          if (j < ncnt) prefetch_l1(j < nna ? a.own + nla + j : a.rest + nlb + (j - nna));
-          if (j + 8 < ncnt)
-            prefetch_l1(j + 8 < nna ? a.own + nla + j + 8 : a.rest + nlb + (j + 8 - nna));
-          if (j == 0 && ncnt > 0) prefetch_l2(a.res + pre[g].x);
-        }
-        charge<2 * G, OWN, COUNT>(a, ee, vv, pp, k, ts, tn, wb, N, qn, n_dec, s_lvl0, n_dead,
-                                  n_early);
       }
-      flush_push<OWN>(a, wb, N, qn);
+      flush_push(a, wb, N, qn);
       if (COUNT && k < a.lvl_cap) {
-        unsigned x0 = n_entries - c_ent, x1 = n_dead - c_dead, x2 = n_early - c_early;
+        unsigned x0 = s_work[threadIdx.x].x - c_ent, x1 = n_dead - c_dead, x2 = n_early - c_early;
         for (int o = 16; o >= 1; o >>= 1) {
           x0 += __shfl_down_sync(TR_FULL, x0, o);
           x1 += __shfl_down_sync(TR_FULL, x1, o);
@@ -594,20 +716,13 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
           atomicAdd(&a.lvl[3 * k + 2], (unsigned long long)x2);
         }
       }
-      if (!grid_barrier(&ctl->bar, &ctl->err, a.wait_ns)) return;
+      if (!phase_end(a, ph, &nCur, nullptr, nullptr)) return;
       ph++;
-      prefetch(N);
-      const int64_t nN = (int64_t)__ldcg(qn);
       s++;
       if (leader) ctl->subrounds++;
-      if (nN == 0) break;
-      { int4 *t = F; F = N; N = t; }
-      nCur = nN > a.item_cap ? a.item_cap : nN;
-      if (nN > a.item_cap && leader) atomicExch(&ctl->err, TRUSS_ECHECK);
-    }
-    if (leader) {
-      ctl->levels++;
-      ctl->kmax = k;
+      if (nCur == 0) break;
+      rev = !rev;
+      nCur = clamp(nCur);
     }
     k++;
   }
@@ -616,10 +731,10 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
     a.trace[ctl->ntrace++] = make_int4(k, -2, (int)(uint32_t)t, (int)(uint32_t)(t >> 32));
   }
   // totals (one atomic per warp)
+  unsigned n_entries = s_work[threadIdx.x].x, n_dec = s_work[threadIdx.x].y;
   for (int o = 16; o >= 1; o >>= 1) {
     n_entries += __shfl_down_sync(TR_FULL, n_entries, o);
     n_dec += __shfl_down_sync(TR_FULL, n_dec, o);
-    n_scan += __shfl_down_sync(TR_FULL, n_scan, o);
     if (COUNT) {
       n_dead += __shfl_down_sync(TR_FULL, n_dead, o);
       n_early += __shfl_down_sync(TR_FULL, n_early, o);
@@ -628,7 +743,6 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
   if (lane == 0) {
     atomicAdd(&ctl->entries, (unsigned long long)n_entries);
     atomicAdd(&ctl->decrements, (unsigned long long)n_dec);
-    atomicAdd(&ctl->scanned, (unsigned long long)n_scan);
     if (COUNT) {
       atomicAdd(&ctl->dead, (unsigned long long)n_dead);
       atomicAdd(&ctl->dead_earlier, (unsigned long long)n_early);
@@ -640,20 +754,16 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
 // decrements it can receive (at most its support) leave it out of reach.
 constexpr int kPinnedRes = INT_MAX / 4;
 
-__global__ void k_peel_init(int64_t m, const int32_t *sup, const uint8_t *pinned, int32_t *res,
-                            uint16_t *stamp, int32_t *alive, int32_t *truss, PeelCtl *ctl) {
+__global__ void k_peel_init(int64_t m, const int32_t *sup, const uint8_t *pinned, uint32_t *word,
+                            int32_t *alive, int32_t *truss, PeelCtl *ctl) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
-    res[e] = (pinned && pinned[e]) ? kPinnedRes : sup[e];
-    stamp[e] = 0;
+    word[e] = (uint32_t)((pinned && pinned[e]) ? kPinnedRes : sup[e]);
     alive[e] = (int32_t)e;
     truss[e] = 0;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    for (int i = 0; i < 3; i++) {
-      ctl->minres[i] = INT_MAX;
-      ctl->live[i] = 0;
-    }
+    for (int i = 0; i < 3; i++) ctl->scan[i].minres = INT_MAX;
   }
 }
 
@@ -805,21 +915,26 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
   const int64_t m = g.m;
   *out = PeelResult{};
   if (m == 0) return TRUSS_OK;
-  // item offsets carry 42 bits
+  // items carry 32-bit block numbers
   if (so.entries >= kOffLimit || (L.own_cnt && so.records >= kOffLimit)) return TRUSS_EINVAL;
   if (so.entries > 0 && (!L.rest || !L.off || (L.own_cnt && (!L.own || !L.own_off))))
     return TRUSS_EINVAL;
-  // items of one sub-round <= sum over its edges of max(1, ceil(sup / kItem))
-  const int64_t item_cap = m + so.entries / kItem + 64;
-  int32_t *res = A.get<int32_t>(m);
-  uint16_t *stamp = A.get<uint16_t>(m);
+  // Items of all edges: the lists in `rest` follow one another, so they touch
+  // at most one block each beyond the array's own; an own part of c entries
+  // touches at most c / kItem + 2.
+  const bool own = L.own_cnt != nullptr;
+  const int64_t item_cap = so.entries / kItem + (own ? 3 : 1) * m + 64;
+  // items are counted in 32 bits: beyond that their queue alone takes 34 GB
+  // and the lists 275 GB or more
+  if (item_cap > (int64_t)UINT32_MAX / 2) return TRUSS_ENOMEM;
+  uint32_t *word = A.get<uint32_t>(m);
   int32_t *al0 = A.get<int32_t>(m), *al1 = A.get<int32_t>(m);
-  int4 *Q0 = A.get<int4>(item_cap), *Q1 = A.get<int4>(item_cap);
+  int4 *Q = A.get<int4>(item_cap);
   PeelCtl *ctl = A.get<PeelCtl>(1);
-  if (!res || !stamp || !al0 || !al1 || !Q0 || !Q1 || !ctl) return TRUSS_ENOMEM;
+  if (!word || !al0 || !al1 || !Q || !ctl) return TRUSS_ENOMEM;
   TR_CUDA(cudaMemsetAsync(ctl, 0, sizeof(PeelCtl), s));
-  k_peel_init<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, so.sup, cfg.pinned, res, stamp, al0,
-                                                          truss, ctl);
+  k_peel_init<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, so.sup, cfg.pinned, word, al0, truss,
+                                                          ctl);
   TR_LAUNCHED();
 
   int dev = 0, sms = cfg.sms;
@@ -829,23 +944,31 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
   // per SM; 3: 1 item per group, one block per SM; otherwise (0, 2) the
   // 64-register kernel with 1 item per group and two blocks per SM
   const int variant = cfg.variant == 1 ? 1 : (cfg.variant == 3 ? 3 : 2);
-  const bool own = L.own_cnt != nullptr;
-  const void *kern;
-  if (cfg.count) {
-    kern = own ? (const void *)k_peel<2, 1, true, true> : (const void *)k_peel<2, 1, false, true>;
-  } else if (own) {
-    kern = variant == 1   ? (const void *)k_peel<1, 2, true>
-           : variant == 3 ? (const void *)k_peel<1, 1, true>
-                          : (const void *)k_peel<2, 1, true>;
-  } else {
-    kern = variant == 1   ? (const void *)k_peel<1, 2, false>
-           : variant == 3 ? (const void *)k_peel<1, 1, false>
-                          : (const void *)k_peel<2, 1, false>;
-  }
+  const void *kern = cfg.count      ? (const void *)k_peel<2, 1, true>
+                     : variant == 1 ? (const void *)k_peel<1, 2>
+                     : variant == 3 ? (const void *)k_peel<1, 1>
+                                    : (const void *)k_peel<2, 1>;
   int occ = 0;
   TR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kPeelBlock, 0));
   if (occ < 1) return TRUSS_ECUDA;
   if (variant != 2 && !cfg.count && occ > 1) occ = 1;
+  // SMs to use: a sub-round of a small graph is a chain of dependent round
+  // trips whatever the grid, and fewer blocks meet sooner.  Up to kWideWork
+  // units of work (list entries and 8 per edge, for the scans) at most half
+  // the SMs, down to kFewSms, at kSmWork units each.  Measured (ms, SMs:
+  // 24 / 38 / 76 / 152), R-MAT of 65 K rows 1.54 / 1.54 / 1.58 / 1.66, 262 K
+  // 3.14 / 3.05 / 3.03 / 3.21, 524 K 4.54 / 4.26 / 4.09 / 4.24, 2.1 M 9.76 /
+  // 8.29 / 7.00 / 6.92; Chung-Lu of 3 M rows 11.1 / 10.3 / 9.75 / 10.2, 10 M
+  // 32.2 / 27.8 / 24.2 / 24.1.  The other half is free for other streams.
+  constexpr int kFewSms = 24;
+  constexpr int64_t kSmWork = 250000, kWideWork = 80000000;
+  const int64_t work = so.entries + 8 * m;
+  if (variant == 2 && work < kWideWork) {
+    const int64_t want = work / kSmWork > kFewSms ? work / kSmWork : kFewSms;
+    if (sms > 2 * kFewSms && want < sms / 2) sms = (int)want;
+    else if (sms > 2 * kFewSms) sms = sms / 2;
+  }
+  if (cfg.max_sms > 0 && sms > cfg.max_sms) sms = cfg.max_sms;
   PeelArgs a{};
   a.m = m;
   a.sup = so.sup;
@@ -854,8 +977,7 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
   a.own_cnt = L.own_cnt;
   a.rest = L.rest;
   a.off = L.off ? L.off : so.toff;
-  a.res = res;
-  a.stamp = stamp;
+  a.word = word;
   a.retag = kRetagMax;
   if (const char *rt = getenv("TRUSS_PEEL_RETAG")) {  // testing: rewrite tags more often
     const int v = atoi(rt);
@@ -864,9 +986,8 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
   a.truss = truss;
   a.alive0 = al0;
   a.alive1 = al1;
-  a.Q0 = Q0;
-  a.Q1 = Q1;
-  a.item_cap = item_cap;
+  a.Q = Q;
+  a.item_cap = (uint32_t)item_cap;
   a.ctl = ctl;
   a.wait_ns = cfg.wait_ns;
   a.k_stop = cfg.k_stop;

@@ -111,7 +111,7 @@ __device__ __forceinline__ int queue_items(const AsyncArgs &a, bool push, int p)
       const int64_t off = lbo + start;
       a.Q[idx] = make_int4(po, cnt, (int)(uint32_t)off, (int)(uint32_t)((uint64_t)off >> 32));
     } else if (t < tot) {
-      atomicExch(&a.ctl->err, TRUSS_ECHECK);
+      raise_error(&a.ctl->bar, &a.ctl->err, TRUSS_ECHECK);
     }
   }
   __threadfence();
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_peel_async(AsyncArgs a) {
         bool late = false;
         if (lane == 0) late = (long long)(global_ns() - t0) > a.wait_ns;
         if (__shfl_sync(TR_FULL, late, 0)) {
-          if (lane == 0) atomicExch(&ctl->err, TRUSS_ETIMEOUT);
+          if (lane == 0) raise_error(&ctl->bar, &ctl->err, TRUSS_ETIMEOUT);
           break;
         }
         if (*(volatile int *)&ctl->err != 0) break;
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_peel_async(AsyncArgs a) {
         if (v[q]) {
           if ((uint32_t)pp[q].x >= (uint32_t)a.m || (uint32_t)pp[q].y >= (uint32_t)a.m ||
               (int64_t)tid[q] >= a.ntri) {
-            atomicExch(&ctl->err, TRUSS_ECHECK);
+            raise_error(&ctl->bar, &ctl->err, TRUSS_ECHECK);
           } else {
             const unsigned bit = 1u << (tid[q] & 31u);
             chg[q] = (atomicOr(&a.dbits[tid[q] >> 5], bit) & bit) == 0u;
