@@ -606,7 +606,7 @@ int run_upper_bound(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src,
   st.triangles = so.entries / 3;
   int32_t *psi = A.get<int32_t>(g.m);
   if (!psi) return TRUSS_ENOMEM;
-  TR_TRY(tr::compute_psi(A, g, so.sup, psi, s));
+  TR_TRY(tr::compute_psi(A, g, so, psi, s));
   OutBuf os, op;
   TR_TRY(stage_out(A, support_out, rows, &os));
   TR_TRY(stage_out(A, psi_out, rows, &op));
@@ -663,7 +663,7 @@ int run_top(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src, const i
   int32_t *cs = A.get<int32_t>(g.m), *cd = A.get<int32_t>(g.m), *ce = A.get<int32_t>(g.m);
   int32_t *phi_rows = A.get<int32_t>(g.m);
   if (!psi || !top || !cs || !cd || !ce || !phi_rows) return TRUSS_ENOMEM;
-  TR_TRY(tr::compute_psi(A, g, so.sup, psi, s));
+  TR_TRY(tr::compute_psi(A, g, so, psi, s));
   std::vector<int64_t> cnt_ge;
   TR_TRY(tr::psi_counts(A, g.m, psi, &cnt_ge, s));
   sg.mark();  // 1: build, support, psi

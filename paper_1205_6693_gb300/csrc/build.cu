@@ -184,6 +184,9 @@ int build_csr(Arena &A, const RowsIn &in, Csr *out, int32_t *d_err, cudaStream_t
     }
     out->m = 0;
     out->order = order;
+    out->sdeg = A.get<int32_t>(n);
+    if (!out->sdeg) return TRUSS_ENOMEM;
+    TR_CUDA(cudaMemsetAsync(out->sdeg, 0, sizeof(int32_t) * (n > 0 ? n : 1), s));
     out->adjp = A.get<int32_t>(1);
     out->esrc = A.get<int32_t>(1);
     return TRUSS_OK;
@@ -243,6 +246,7 @@ int build_csr(Arena &A, const RowsIn &in, Csr *out, int32_t *d_err, cudaStream_t
   TR_TRY(sort_pairs_u32(tmp, &tb, (const uint32_t *)deg, (uint32_t *)sdeg, ids, order, n, 0, db,
                         s));
   out->order = order;
+  out->sdeg = sdeg;
   k_newid<<<grid_for(n, kBlock, maxg), kBlock, 0, s>>>(n, order, newid);
   TR_LAUNCHED();
 

@@ -17,12 +17,14 @@
 //        not in the k+1-core).  Vertices removed together need no exchange:
 //        a neighbour in the same frontier is simply skipped.
 //
-// Vertex state is stamp[v]: 0 = alive, s = in the frontier of sub-round s,
-// 0 < stamp < s = removed earlier; a vertex pushed during sub-round s is
-// stamped s+1 and still counts as alive during s.  Neighbours come from a
-// symmetric adjacency built from the oriented CSR.  A frontier vertex is
-// split into work items of kItem neighbours, as in the edge peel, so a
-// warp's share of a sub-round is bounded whatever the degrees.
+// Vertex state is one word, the current degree, with the top bit set once the
+// vertex is removed: a neighbour costs one read and, if alive, one decrement.
+// A vertex marked while others still decrement it only loses counts that no
+// longer matter (its degree stays >= 0: every neighbour is removed once).
+// Neighbours come from a symmetric adjacency built from the oriented CSR.  A
+// frontier vertex is split into work items of kItem neighbours, as in the
+// edge peel, so a warp's share of a sub-round is bounded whatever the degrees.
+// Phases end as in the edge peel (phase_end).  R-MAT scale 20: CORE_FIG.
 #include <climits>
 
 #include "engine.h"
@@ -37,14 +39,7 @@ constexpr int kItem = 16;  // neighbours per work item (8 lanes x 2)
 constexpr int kWQ = 64;    // work items staged per warp
 constexpr int kWA = 128;   // alive-list entries staged per warp
 
-struct CoreCtl {
-  unsigned long long bar;
-  int err;
-  int pad0;
-  unsigned long long qf[3];  // frontier items appended in phase p (slot p % 3)
-  unsigned long long qa[3];  // alive-list entries appended in phase p
-  int minres[3];             // per scan (slot = scan index % 3)
-  int live[3];
+struct CoreCtl : PhaseCtl {
   int levels, subrounds, kmax, pad1;
 };
 
@@ -52,15 +47,16 @@ struct CoreArgs {
   int64_t n;
   const int64_t *soff;  // [n+1] symmetric adjacency offsets
   const int32_t *sadj;  // [2m]
-  int32_t *deg;         // current degrees (start: full degrees)
-  int32_t *stamp;
+  uint32_t *word;       // current degree; kGone set once removed
   int32_t *core;
   int32_t *alive0, *alive1;
   int4 *Q0, *Q1;  // work items (v, cnt | first << 8, offset lo, hi)
-  int64_t item_cap;
+  uint32_t item_cap;
   CoreCtl *ctl;
   long long wait_ns;
 };
+
+constexpr uint32_t kGone = 0x80000000u;
 
 __device__ __forceinline__ int items_of(int len) { return len > 0 ? (len + kItem - 1) / kItem : 1; }
 
@@ -75,9 +71,9 @@ __device__ __forceinline__ void flush_items(const CoreArgs &a, WarpBuf &wb, int4
                                             unsigned long long *qctr) {
   if (wb.ni == 0) return;
   const int lane = lane_id();
-  unsigned long long b = 0;
-  if (lane == 0) b = atomicAdd(qctr, (unsigned long long)wb.ni);
-  const long long b0 = (long long)__shfl_sync(TR_FULL, b, 0);
+  uint32_t b = 0;
+  if (lane == 0) b = reserve_items(qctr, wb.ni);
+  const uint32_t b0 = __shfl_sync(TR_FULL, b, 0);
   for (int t = lane; t < wb.ni; t += 32)
     if (b0 + t < a.item_cap) Q[b0 + t] = wb.items[t];
   __syncwarp();
@@ -85,12 +81,12 @@ __device__ __forceinline__ void flush_items(const CoreArgs &a, WarpBuf &wb, int4
 }
 
 __device__ __forceinline__ void flush_alive(const CoreArgs &a, WarpBuf &wb, int32_t *A2,
-                                            unsigned long long *actr) {
+                                            int *actr) {
   if (wb.na == 0) return;
   const int lane = lane_id();
-  unsigned long long b = 0;
-  if (lane == 0) b = atomicAdd(actr, (unsigned long long)wb.na);
-  const long long b0 = (long long)__shfl_sync(TR_FULL, b, 0);
+  int b = 0;
+  if (lane == 0) b = atomicAdd(actr, wb.na);
+  const int b0 = __shfl_sync(TR_FULL, b, 0);
   for (int t = lane; t < wb.na; t += 32)
     if (b0 + t < a.n) A2[b0 + t] = wb.alive[t];
   __syncwarp();
@@ -98,7 +94,7 @@ __device__ __forceinline__ void flush_alive(const CoreArgs &a, WarpBuf &wb, int3
 }
 
 __device__ __forceinline__ void push_alive(const CoreArgs &a, bool keep, int v, WarpBuf &wb,
-                                           int32_t *A2, unsigned long long *actr) {
+                                           int32_t *A2, int *actr) {
   const unsigned mask = __ballot_sync(TR_FULL, keep);
   if (mask == 0) return;
   const int tot = __popc(mask);
@@ -108,10 +104,9 @@ __device__ __forceinline__ void push_alive(const CoreArgs &a, bool keep, int v, 
   wb.na += tot;
 }
 
-// Append the work items of vertex p (lanes with `push`), stamping it.  All
-// lanes call it.  Batches larger than the staging buffer go straight to Q.
+// Append the work items of vertex p (lanes with `push`).  All lanes call it.  Batches larger than the staging buffer go straight to Q.
 __device__ __forceinline__ void push_items(const CoreArgs &a, bool push, int p, WarpBuf &wb,
-                                           int4 *Q, unsigned long long *qctr, int stamp_val) {
+                                           int4 *Q, unsigned long long *qctr) {
   const int lane = lane_id();
   int n = 0, L = 0;
   int64_t lb = 0;
@@ -119,24 +114,23 @@ __device__ __forceinline__ void push_items(const CoreArgs &a, bool push, int p, 
     lb = __ldg(&a.soff[p]);
     L = (int)(__ldg(&a.soff[p + 1]) - lb);
     n = items_of(L);
-    a.stamp[p] = stamp_val;
   }
   const int P = warp_incl_scan(n);
   const int tot = __shfl_sync(TR_FULL, P, 31);
   if (tot == 0) return;
   int4 *dst;
-  long long b0;
+  uint32_t b0;
   if (tot > kWQ) {
-    unsigned long long b = 0;
-    if (lane == 31) b = atomicAdd(qctr, (unsigned long long)tot);
-    b0 = (long long)__shfl_sync(TR_FULL, b, 31);
+    uint32_t b = 0;
+    if (lane == 31) b = reserve_items(qctr, tot);
+    b0 = __shfl_sync(TR_FULL, b, 31);
     dst = Q;
   } else {
     if (wb.ni + tot > kWQ) flush_items(a, wb, Q, qctr);
     b0 = wb.ni;
     dst = wb.items;
   }
-  const long long lim = tot > kWQ ? a.item_cap : (long long)kWQ;
+  const uint32_t lim = tot > kWQ ? a.item_cap : (uint32_t)kWQ;
   for (int t0 = 0; t0 < tot; t0 += 32) {
     const int t = t0 + lane;
     const int o = warp_owner(P, t < tot ? t : tot - 1);
@@ -145,7 +139,7 @@ __device__ __forceinline__ void push_items(const CoreArgs &a, bool push, int p, 
     const int no = __shfl_sync(TR_FULL, n, o);
     const int Lo = __shfl_sync(TR_FULL, L, o);
     const int64_t lbo = __shfl_sync(TR_FULL, lb, o);
-    const long long idx = b0 + t;
+    const uint32_t idx = b0 + t;
     if (t < tot && idx < lim) {
       const int it = t - (Po - no);
       const int start = it * kItem;
@@ -162,94 +156,116 @@ __device__ __forceinline__ void push_items(const CoreArgs &a, bool push, int p, 
 __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
   const int lane = lane_id();
   const int wib = threadIdx.x >> 5;
-  const int64_t gwarp = (int64_t)blockIdx.x * kWarps + wib;
-  const int64_t twarps = (int64_t)gridDim.x * kWarps;
+  // consecutive warps of the launch sit in different blocks, so a phase with
+  // little work spreads it over all SMs
+  const uint32_t gwarp = wib * gridDim.x + blockIdx.x;
+  const uint32_t twarps = gridDim.x * kWarps;
   const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
   CoreCtl *ctl = a.ctl;
   __shared__ int4 s_items[kWarps][kWQ];
   __shared__ int32_t s_alive[kWarps][kWA];
-  __shared__ int s_minres, s_live;
+  __shared__ int s_minres, s_live, s_any;
   WarpBuf wb{s_items[wib], 0, s_alive[wib], 0};
   if (threadIdx.x == 0) {
     s_minres = INT_MAX;
     s_live = 0;
+    s_any = 0;
   }
   __syncthreads();
 
-  int k = 0, s = 1, sc = 0;
+  int k = 0, sc = 0;
   unsigned ph = 0;
   int32_t *alive = a.alive0, *alive2 = a.alive1;
   int4 *F = a.Q0, *N = a.Q1;
-  int64_t nAlive = a.n;
+  int nAlive = (int)a.n;
   bool compact = false;
+  auto clamp = [&](uint32_t n) {
+    if (n <= a.item_cap) return n;
+    // appends beyond the queue were dropped
+    if (leader) raise_error(&ctl->phase[ph % 3], &ctl->err, TRUSS_ECHECK);
+    return a.item_cap;
+  };
 
   for (;;) {
     // ------------------------------------------------------------ scan ---
-    const int slot = sc % 3;
-    unsigned long long *qf = &ctl->qf[ph % 3], *qa = &ctl->qa[ph % 3];
+    ScanOut *scan = &ctl->scan[sc % 3];
+    unsigned long long *qf = &ctl->phase[ph % 3];
     if (leader) {
-      ctl->minres[(sc + 1) % 3] = INT_MAX;
-      ctl->live[(sc + 1) % 3] = 0;
-      ctl->qf[(ph + 1) % 3] = 0;
-      ctl->qa[(ph + 1) % 3] = 0;
+      *(int4 *)&ctl->scan[(sc + 1) % 3] = make_int4(INT_MAX, 0, 0, 0);
+      ctl->phase[(ph + 1) % 3] = 0;
     }
-    int wmin = INT_MAX, wlive = 0;
-    for (int64_t base = gwarp * 32; base < nAlive; base += twarps * 32) {
+    int lmin = INT_MAX, llive = 0;  // of this lane
+    bool lany = false;
+    for (int64_t base = (int64_t)gwarp * 32; base < nAlive; base += (int64_t)twarps * 32) {
       const int64_t i = base + lane;
       const int v = i < nAlive ? __ldcg(&alive[i]) : -1;
-      const int st = v >= 0 ? __ldcg(&a.stamp[v]) : 1;
-      const int dv = v >= 0 ? __ldcg(&a.deg[v]) : 0;
-      const bool live = v >= 0 && st == 0;
-      const bool toF = live && dv <= k;
+      const uint32_t w = v >= 0 ? __ldcg(&a.word[v]) : kGone;
+      const bool live = (int32_t)w >= 0;
+      const bool toF = live && (int)w <= k;
       const bool keep = live && !toF;
-      push_items(a, toF, v, wb, F, qf, s);
-      if (compact) push_alive(a, keep, v, wb, alive2, qa);
-      wmin = min(wmin, __reduce_min_sync(TR_FULL, keep ? dv : INT_MAX));
-      wlive += __popc(__ballot_sync(TR_FULL, keep));
+      if (toF) {
+        a.word[v] = kGone | w;
+        lany = true;
+        if (w == 0) a.core[v] = k;  // no neighbour left: no item
+      }
+      push_items(a, toF && w > 0, v, wb, F, qf);
+      if (compact) push_alive(a, keep, v, wb, alive2, &scan->listed);
+      if (keep) {
+        lmin = min(lmin, (int)w);
+        llive++;
+      }
     }
     flush_items(a, wb, F, qf);
-    if (compact) flush_alive(a, wb, alive2, qa);
-    if (lane == 0) {
-      if (wmin != INT_MAX) atomicMin(&s_minres, wmin);
-      if (wlive) atomicAdd(&s_live, wlive);
+    if (compact) flush_alive(a, wb, alive2, &scan->listed);
+    if ((int64_t)gwarp * 32 < nAlive) {
+      lmin = __reduce_min_sync(TR_FULL, lmin);
+      llive = __reduce_add_sync(TR_FULL, llive);
+      const bool wany = __any_sync(TR_FULL, lany);
+      if (lane == 0) {
+        if (lmin != INT_MAX) atomicMin(&s_minres, lmin);
+        if (llive) atomicAdd(&s_live, llive);
+        if (wany) s_any = 1;
+      }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      if (s_minres != INT_MAX) atomicMin(&ctl->minres[slot], s_minres);
-      if (s_live) atomicAdd(&ctl->live[slot], s_live);
+      if (s_minres != INT_MAX) atomicMin(&scan->minres, s_minres);
+      if (s_live) atomicAdd(&scan->live, s_live);
+      if (s_any) scan->any = 1;
       s_minres = INT_MAX;
       s_live = 0;
+      s_any = 0;
     }
-    if (!grid_barrier(&ctl->bar, &ctl->err, a.wait_ns)) return;
+    uint32_t nCur;  // items of the frontier
+    ScanOut found;
+    if (!phase_end(ctl, a.wait_ns, ph, &nCur, scan, &found)) return;
     ph++;
-    const int minres = __ldcg(&ctl->minres[slot]);
-    const int64_t live = __ldcg(&ctl->live[slot]);
-    const int64_t nF = (int64_t)__ldcg(qf);
     if (compact) {
-      nAlive = (int64_t)__ldcg(qa);
+      nAlive = found.listed;
       int32_t *t = alive;
       alive = alive2;
       alive2 = t;
     }
-    compact = 2 * live <= nAlive;
+    compact = 2 * (int64_t)found.live <= nAlive;
     sc++;
-    if (nF == 0) {
-      if (live == 0) break;
-      k = minres;  // every alive vertex has degree >= k+1: skip empty levels
+    if (found.any && leader) {
+      ctl->levels++;
+      ctl->kmax = k;
+    }
+    if (nCur == 0) {
+      // nothing removed had a neighbour left, so the degrees stand
+      if (found.live == 0) break;
+      k = found.minres;  // every alive vertex has degree >= k+1: skip empty levels
       continue;
     }
     // --------------------------------------------------------- sub-rounds ---
-    int64_t nCur = nF > a.item_cap ? a.item_cap : nF;
-    if (nF > a.item_cap && leader) raise_error(&ctl->bar, &ctl->err, TRUSS_ECHECK);
+    nCur = clamp(nCur);
     for (;;) {
-      unsigned long long *qn = &ctl->qf[ph % 3];
-      if (leader) {
-        ctl->qf[(ph + 1) % 3] = 0;
-        ctl->qa[(ph + 1) % 3] = 0;
-      }
+      unsigned long long *qn = &ctl->phase[ph % 3];
+      if (leader) ctl->phase[(ph + 1) % 3] = 0;
       const int grp = lane >> 3, j = lane & 7;
-      for (int64_t base = gwarp * 4; base < nCur; base += twarps * 4) {
-        const int64_t it = base + grp;
+      for (uint32_t base = gwarp * 4; base < nCur; base += twarps * 4) {
+        const uint32_t it = base + grp;
         int v = 0, cnt = 0;
         int64_t lb = 0;
         if (it < nCur) {
@@ -260,7 +276,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
           if ((item.y >> 8) && j == 0) a.core[v] = k;
         }
         int w[2];
-        bool dec[2];
+        uint32_t x[2];
 #pragma unroll
         for (int q = 0; q < 2; q++) {
           const int jj = j + 8 * q;
@@ -268,76 +284,73 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
         }
 #pragma unroll
         for (int q = 0; q < 2; q++) {
-          dec[q] = false;
-          if (w[q] >= 0) {
-            if ((uint32_t)w[q] >= (uint32_t)a.n) {
-              raise_error(&ctl->bar, &ctl->err, TRUSS_ECHECK);
-            } else {
-              const int sw = __ldcg(&a.stamp[w[q]]);
-              dec[q] = sw == 0 || sw > s;  // alive (possibly pushed this sub-round)
-            }
+          if (w[q] >= 0 && (uint32_t)w[q] >= (uint32_t)a.n) {
+            raise_error(&ctl->phase[ph % 3], &ctl->err, TRUSS_ECHECK);
+            w[q] = -1;
           }
+          x[q] = w[q] >= 0 ? __ldcg(&a.word[w[q]]) : kGone;
         }
-        int old[2];
 #pragma unroll
-        for (int q = 0; q < 2; q++) old[q] = dec[q] ? atomicSub(&a.deg[w[q]], 1) : INT_MIN;
+        for (int q = 0; q < 2; q++)
+          x[q] = (int32_t)x[q] >= 0 ? atomicSub(&a.word[w[q]], 1u) : kGone;
         // one push_items site: each step pushes one pending neighbour per lane
-        unsigned pend = (old[0] == k + 1 ? 1u : 0u) | (old[1] == k + 1 ? 2u : 0u);
+        unsigned pend = (x[0] == (uint32_t)(k + 1) ? 1u : 0u) | (x[1] == (uint32_t)(k + 1) ? 2u : 0u);
         while (__any_sync(TR_FULL, pend != 0)) {
           const bool has = pend != 0;
           const int b = has ? __ffs(pend) - 1 : 0;
           pend &= pend - 1;
-          push_items(a, has, b ? w[1] : w[0], wb, N, qn, s + 1);
+          const int q = b ? w[1] : w[0];
+          if (has) atomicOr(&a.word[q], kGone);  // others may still decrement it
+          push_items(a, has, q, wb, N, qn);
         }
       }
       flush_items(a, wb, N, qn);
-      if (!grid_barrier(&ctl->bar, &ctl->err, a.wait_ns)) return;
+      if (!phase_end(ctl, a.wait_ns, ph, &nCur, nullptr, nullptr)) return;
       ph++;
-      const int64_t nN = (int64_t)__ldcg(qn);
-      s++;
       if (leader) ctl->subrounds++;
-      if (nN == 0) break;
+      if (nCur == 0) break;
       { int4 *t = F; F = N; N = t; }
-      nCur = nN > a.item_cap ? a.item_cap : nN;
-      if (nN > a.item_cap && leader) raise_error(&ctl->bar, &ctl->err, TRUSS_ECHECK);
-    }
-    if (leader) {
-      ctl->levels++;
-      ctl->kmax = k;
+      nCur = clamp(nCur);
     }
     k++;
   }
 }
 
-// Symmetric degrees: out-degree plus in-degree of every vertex.
-__global__ void k_sym_deg(int64_t n, int64_t m, const int64_t *offp, const int32_t *adjp,
-                          unsigned long long *sdeg) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
-       e += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&sdeg[adjp[e]], 1ull);
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&sdeg[v], (unsigned long long)(offp[v + 1] - offp[v]));
+__global__ void k_widen(int64_t n, const int32_t *x, int64_t *y) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    y[i] = i < n ? x[i] : 0;
 }
 
-// sadj[soff[v] ..) = all neighbours of v, in any order.
-__global__ void k_sym_fill(int64_t m, const int32_t *esrc, const int32_t *adjp,
-                           const int64_t *soff, unsigned long long *cur, int32_t *sadj) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int u = esrc[e], v = adjp[e];
-    sadj[soff[u] + (int64_t)atomicAdd(&cur[u], 1ull)] = v;
-    sadj[soff[v] + (int64_t)atomicAdd(&cur[v], 1ull)] = u;
+// sadj[soff[v] ..) = v's out-neighbours, then its in-neighbours in any order.
+// Out-neighbours are where they are in adjp; in-neighbours take a cursor, one
+// atomic per group of lanes of a warp with the same head (one per edge and
+// end, hubs included, took 574 us on R-MAT scale 20, now FILL_FIG us).
+__global__ void k_sym_fill(int64_t m, const int64_t *offp, const int32_t *esrc,
+                           const int32_t *adjp, const int64_t *soff, int32_t *cur,
+                           int32_t *sadj) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const unsigned lt = (1u << lane_id()) - 1u;
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < m; b += stride) {
+    const int64_t e = b + threadIdx.x;
+    const bool ok = e < m;
+    const int u = ok ? esrc[e] : 0, v = ok ? adjp[e] : -1;
+    if (ok) sadj[soff[u] + (e - offp[u])] = v;
+    const unsigned peers = __match_any_sync(TR_FULL, v);
+    const int first = __ffs(peers) - 1;
+    int c = 0;
+    if (ok && lane_id() == first) c = atomicAdd(&cur[v], __popc(peers));
+    c = __shfl_sync(TR_FULL, c, first);
+    if (ok) sadj[soff[v] + (offp[v + 1] - offp[v]) + c + __popc(peers & lt)] = u;
   }
 }
 
-__global__ void k_core_init(int64_t n, const int64_t *soff, int32_t *deg, int32_t *stamp,
-                            int32_t *alive, CoreCtl *ctl) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->minres[0] = INT_MAX;  // first scan's slot
+__global__ void k_core_init(int64_t n, const int32_t *sdeg, uint32_t *word, int32_t *alive,
+                            CoreCtl *ctl) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->scan[0].minres = INT_MAX;  // first scan's slot
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    deg[v] = (int32_t)(soff[v + 1] - soff[v]);
-    stamp[v] = 0;
+    word[v] = (uint32_t)sdeg[v];
     alive[v] = (int32_t)v;
   }
 }
@@ -358,33 +371,34 @@ int run_core(Arena &A, const Csr &g, int sms, long long wait_ns, int32_t *core_o
   *kmax = 0;
   *levels = *subrounds = 0;
   if (n == 0) return TRUSS_OK;
-  unsigned long long *cnt = A.get<unsigned long long>(n + 1);
-  int64_t *soff = A.get<int64_t>(n + 1);
+  int32_t *cur = A.get<int32_t>(n);
+  int64_t *deg64 = A.get<int64_t>(n + 1), *soff = A.get<int64_t>(n + 1);
   int32_t *sadj = A.get<int32_t>(2 * m);
-  int32_t *deg = A.get<int32_t>(n), *stamp = A.get<int32_t>(n), *core = A.get<int32_t>(n);
+  uint32_t *word = A.get<uint32_t>(n);
+  int32_t *core = A.get<int32_t>(n);
   int32_t *al0 = A.get<int32_t>(n), *al1 = A.get<int32_t>(n);
   // every vertex is pushed at most once; its items number at most
-  // deg / kItem + 1, so 2m / kItem + n items bound any frontier
+  // deg / kItem + 1, so 2m / kItem + n items bound any frontier (below 2^32)
   const int64_t item_cap = 2 * m / kItem + n + 1;
   int4 *Q0 = A.get<int4>(item_cap), *Q1 = A.get<int4>(item_cap);
   CoreCtl *ctl = A.get<CoreCtl>(1);
-  if (!cnt || !soff || !sadj || !deg || !stamp || !core || !al0 || !al1 || !Q0 || !Q1 || !ctl)
+  if (!cur || !deg64 || !soff || !sadj || !word || !core || !al0 || !al1 || !Q0 || !Q1 || !ctl)
     return TRUSS_ENOMEM;
-  TR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * (n + 1), s));
-  k_sym_deg<<<grid_for(m > n ? m : n, 256, 152 * 16), 256, 0, s>>>(n, m, g.offp, g.adjp, cnt);
+  k_widen<<<grid_for(n + 1, 256, 152 * 16), 256, 0, s>>>(n, g.sdeg, deg64);
   TR_LAUNCHED();
   size_t tb = 0;
-  TR_TRY(exclusive_sum_i64(nullptr, &tb, (const int64_t *)cnt, soff, n + 1, s));
+  TR_TRY(exclusive_sum_i64(nullptr, &tb, deg64, soff, n + 1, s));
   void *tmp = A.alloc(tb);
   if (!tmp) return TRUSS_ENOMEM;
-  TR_TRY(exclusive_sum_i64(tmp, &tb, (const int64_t *)cnt, soff, n + 1, s));
-  TR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * (n + 1), s));
+  TR_TRY(exclusive_sum_i64(tmp, &tb, deg64, soff, n + 1, s));
+  TR_CUDA(cudaMemsetAsync(cur, 0, sizeof(int32_t) * n, s));
   if (m > 0) {
-    k_sym_fill<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, g.esrc, g.adjp, soff, cnt, sadj);
+    k_sym_fill<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, g.offp, g.esrc, g.adjp, soff, cur,
+                                                           sadj);
     TR_LAUNCHED();
   }
   TR_CUDA(cudaMemsetAsync(ctl, 0, sizeof(CoreCtl), s));
-  k_core_init<<<grid_for(n, 256, 152 * 16), 256, 0, s>>>(n, soff, deg, stamp, al0, ctl);
+  k_core_init<<<grid_for(n, 256, 152 * 16), 256, 0, s>>>(n, g.sdeg, word, al0, ctl);
   TR_LAUNCHED();
   int occ = 0;
   TR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_core, kBlock, 0));
@@ -394,14 +408,13 @@ int run_core(Arena &A, const Csr &g, int sms, long long wait_ns, int32_t *core_o
   a.n = n;
   a.soff = soff;
   a.sadj = sadj;
-  a.deg = deg;
-  a.stamp = stamp;
+  a.word = word;
   a.core = core;
   a.alive0 = al0;
   a.alive1 = al1;
   a.Q0 = Q0;
   a.Q1 = Q1;
-  a.item_cap = item_cap;
+  a.item_cap = (uint32_t)item_cap;
   a.ctl = ctl;
   a.wait_ns = wait_ns;
   void *args[] = {&a};

@@ -99,6 +99,7 @@ struct Csr {
   int32_t *esrc = nullptr;   // [m]   tail (lower-ranked endpoint) of edge e
   int32_t *row2e = nullptr;  // [rows] row -> e, -1 for self-loop rows
   int32_t *order = nullptr;  // [n]   rank -> input vertex id
+  int32_t *sdeg = nullptr;   // [n]   degree of the vertex of each rank (ascending)
 };
 
 struct DevCounters;  // device scratch for small counters (api.cu)
@@ -226,7 +227,7 @@ int batch_graph_counts(const Csr &g, int32_t G, const int64_t *voff, const int32
 // ------------------------------------------------------------ top-t ---
 // psi(e) = min{sup(e), x_u, x_v} + 2 of every edge (Procedure 6 with the
 // whole graph as H) (topt.cu).
-int compute_psi(Arena &A, const Csr &g, const int32_t *sup, int32_t *psi, cudaStream_t s);
+int compute_psi(Arena &A, const Csr &g, const SupportOut &so, int32_t *psi, cudaStream_t s);
 // Largest psi and the count of edges with psi >= k for k = 0 .. max psi
 // (host vector, cnt_ge[k]).
 int psi_counts(Arena &A, int64_t m, const int32_t *psi, std::vector<int64_t> *cnt_ge,

@@ -92,28 +92,11 @@ constexpr int kItem = 16;  // list entries per work item (8 lanes x 2)
 constexpr int kWP = 32;    // pushed edges staged per warp (one per lane)
 constexpr int kWA = 128;   // alive-list entries staged per warp
 
-// What a scan found (slot = scan index % 3).
-struct __align__(16) ScanOut {
-  int minres;  // least residual of the edges left alive
-  int live;    // how many
-  int any;     // non-zero: the scan removed an edge
-  int listed;  // entries of the rewritten alive list
-};
-
-struct PeelCtl {
-  // Phase p (slot p % 3): barrier arrivals (bits 0 .. 15), frontier items
-  // appended (16 .. 62); top bit: some block has recorded an error.
-  unsigned long long phase[3];
-  int err;
-  int pad0;
-  ScanOut scan[3];
+struct PeelCtl : PhaseCtl {
   int levels, subrounds, kmax, ntrace;
   unsigned long long entries, decrements, scanned;
   unsigned long long dead, dead_earlier;  // counting runs
 };
-
-constexpr int kItemShift = 16;
-constexpr unsigned long long kArriveMask = (1ull << kItemShift) - 1;
 
 struct PeelArgs {
   int64_t m;
@@ -199,11 +182,6 @@ struct Queue {
   bool rev;
   __device__ __forceinline__ int4 *at(uint32_t i) const { return Q + (rev ? cap - 1 - i : i); }
 };
-
-// Reserve n items of phase word *w; the index of the first.
-__device__ __forceinline__ uint32_t reserve_items(unsigned long long *w, int n) {
-  return (uint32_t)(atomicAdd(w, (unsigned long long)(unsigned)n << kItemShift) >> kItemShift);
-}
 
 // Expand the staged pushed edges into work items and append them to queue Q
 // with one reservation.  The list length and offsets of all staged edges
@@ -317,46 +295,6 @@ __device__ __forceinline__ bool is_dead(uint32_t w, uint32_t fs, uint32_t fn) {
   return (int32_t)w < 0 && h != fs && h != fn;
 }
 
-// End of a phase: a barrier of the whole grid, after which *items is the number of items the phase appended and, for a
-// scan, *so is what it found.  The count shares its word with the barrier's
-// arrivals, so the load that sees the last arrival brings it along, and one
-// thread per block reads and passes it on: read by every warp, one L2 sector
-// served 4,864 requests per value and barrier (1.1 us of each sub-round, 5
-// to 7 us of each scan).  A grid barrier that waits longer than wait_ns
-// records TRUSS_ETIMEOUT.  Returns false if some block has recorded an error.
-__device__ __forceinline__ bool phase_end(const PeelArgs &a, unsigned ph, uint32_t *items,
-                                          const ScanOut *scan, ScanOut *so) {
-  __shared__ unsigned long long s_word2[2];  // by phase parity: read until the next phase ends
-  __shared__ ScanOut s_scan2[2];
-  unsigned long long &s_word = s_word2[ph & 1];
-  ScanOut &s_scan = s_scan2[ph & 1];
-  unsigned long long *w = &a.ctl->phase[ph % 3];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long v = atom_add_acq_rel_gpu(w, 1ull) + 1;
-    if ((v & kArriveMask) != gridDim.x) {
-      const unsigned long long t0 = global_ns();
-      for (unsigned spins = 1;; spins++) {
-        v = ld_acquire_gpu(w);
-        if ((v & kArriveMask) == gridDim.x || (v & kBarErr)) break;
-        if (spins > 32) __nanosleep(32);
-        if ((spins & 15) == 0 && (long long)(global_ns() - t0) > a.wait_ns) {
-          raise_error(w, &a.ctl->err, TRUSS_ETIMEOUT);
-          v = kBarErr;
-          break;
-        }
-      }
-    }
-    s_word = v;
-    if (scan) *(int4 *)&s_scan = __ldcg((const int4 *)scan);
-  }
-  __syncthreads();
-  const unsigned long long v = s_word;
-  *items = (uint32_t)((v & ~kBarErr) >> kItemShift);
-  if (scan) *so = s_scan;
-  return (v & kBarErr) == 0;
-}
-
 // MINB = resident blocks per SM the register budget is sized for (1: up to
 // 128 registers per thread, 2: 64); G = work items per 8-lane group per
 // iteration (2 entries per lane per item).
@@ -416,7 +354,7 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
         a.word[e] = gone_tag(kDead) | (w & kResMax);
     }
     uint32_t items;
-    const bool ok = phase_end(a, ph, &items, nullptr, nullptr);
+    const bool ok = phase_end(ctl, a.wait_ns, ph, &items, nullptr, nullptr);
     ph++;
     return ok;
   };
@@ -518,7 +456,7 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
     }
     uint32_t nCur;  // items of the frontier
     ScanOut found;
-    if (!phase_end(a, ph, &nCur, scan, &found)) return;
+    if (!phase_end(ctl, a.wait_ns, ph, &nCur, scan, &found)) return;
     ph++;
     const int minres = found.minres, live = found.live, any = found.any;
     if (leader) ctl->scanned += (unsigned)nAlive;
@@ -716,7 +654,7 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
           atomicAdd(&a.lvl[3 * k + 2], (unsigned long long)x2);
         }
       }
-      if (!phase_end(a, ph, &nCur, nullptr, nullptr)) return;
+      if (!phase_end(ctl, a.wait_ns, ph, &nCur, nullptr, nullptr)) return;
       ph++;
       s++;
       if (leader) ctl->subrounds++;

@@ -458,11 +458,13 @@ __global__ void __launch_bounds__(kBlock, 3) k_support_v(SupVArgs a) {
   }
 }
 
-// Edges grouped by head: counts, then a fill with one cursor per head.
-__global__ void k_head_count(int64_t m, const int32_t *adjp, unsigned long long *cnt) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
-       e += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&cnt[adjp[e]], 1ull);
+// In-degree of every rank: its degree less its out-degree (entry n is 0).  (A
+// counter per head, one atomic per edge, serialised on the hubs: 325 us of
+// 10 M Chung-Lu rows, 1,046 us of 42 M; this pass reads n words.)
+__global__ void k_in_degree(int64_t n, const int32_t *sdeg, const int64_t *offp, int64_t *cnt) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v <= n;
+       v += (int64_t)gridDim.x * blockDim.x)
+    cnt[v] = v < n ? (int64_t)sdeg[v] - (offp[v + 1] - offp[v]) : 0;
 }
 
 __global__ void k_seq(int64_t m, int32_t *x) {
@@ -602,6 +604,7 @@ constexpr int kLBlock = 512;
 constexpr int kLCap = 16384;       // shared cursor counters per range (64 KB)
 constexpr int kLEdgeCost = 4;      // range cost per edge (next to its records)
 constexpr int64_t kLRangeCost = (int64_t)kLCap * kLEdgeCost / 2;
+constexpr int64_t kLMinCost = 512;
 
 struct ListPass {
   int64_t m, n;
@@ -738,17 +741,17 @@ __global__ void k_list_costs(int64_t m, const int32_t *cuv, const int32_t *inedg
   }
 }
 
-// vb[r] = first vertex v with cost(v) >= r * kLRangeCost, for r < nr, and
-// vb[nr] = n; cost(v) = pre[idx[v]] (+ kLEdgeCost * offp[v] for pass 2).
+// vb[r] = first vertex v with cost(v) >= r * cost, for r < nr, and vb[nr] =
+// n; cost(v) = pre[idx[v]] (+ kLEdgeCost * offp[v] for pass 2).
 __global__ void k_list_ranges(int64_t n, int64_t nr, const int64_t *pre, const int64_t *idx,
-                              const int64_t *offp, bool head, int64_t *vb) {
+                              const int64_t *offp, bool head, int64_t cost, int64_t *vb) {
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r <= nr;
        r += (int64_t)gridDim.x * blockDim.x) {
     if (r == nr) {
       vb[r] = n;
       continue;
     }
-    const int64_t x = r * kLRangeCost;
+    const int64_t x = r * cost;
     int64_t lo = 0, hi = n;
     while (lo < hi) {
       const int64_t mid = (lo + hi) >> 1;
@@ -879,7 +882,7 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, 
   int64_t *sup64 = A.get<int64_t>(m + 1), *toff = A.get<int64_t>(m + 1);
   int64_t *wcost = A.get<int64_t>(m + 1), *wpre = A.get<int64_t>(m + 1);
   int64_t *wbound = A.get<int64_t>(m + 1), *tbpre = A.get<int64_t>(m + 1);
-  unsigned long long *hcnt = A.get<unsigned long long>(n + 1);
+  int64_t *hcnt = A.get<int64_t>(n + 1);
   int64_t *inoff = A.get<int64_t>(n + 1);
   int32_t *inedge = A.get<int32_t>(m), *ihead = A.get<int32_t>(m);
   if (!supA || !supB || !sup || !sup64 || !toff || !wcost || !wpre || !wbound || !tbpre ||
@@ -889,18 +892,17 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, 
   TR_CUDA(cudaMemsetAsync(supB, 0, sizeof(int32_t) * m, s));
   int64_t W = 0, R = 0;
   if (m > 0) {
-    // edges grouped by head: counts and their prefix give each head's
+    // edges grouped by head: in-degrees and their prefix give each head's
     // group; a stable radix sort of (head, edge id) fills the groups in
     // edge order (the edge ids sit in wcost's memory until the sort)
-    TR_CUDA(cudaMemsetAsync(hcnt, 0, sizeof(unsigned long long) * (n + 1), s));
-    k_head_count<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, g.adjp, hcnt);
+    k_in_degree<<<grid_for(n + 1, 256, 152 * 16), 256, 0, s>>>(n, g.sdeg, g.offp, hcnt);
     TR_LAUNCHED();
     int32_t *ids = (int32_t *)wcost;
     k_seq<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, ids);
     TR_LAUNCHED();
     const int hbits = bits_for((uint64_t)(n > 1 ? n - 1 : 1));
     size_t tb = 0, tb2 = 0, tb3 = 0;
-    TR_TRY(exclusive_sum_i64(nullptr, &tb, (const int64_t *)hcnt, inoff, n + 1, s));
+    TR_TRY(exclusive_sum_i64(nullptr, &tb, hcnt, inoff, n + 1, s));
     TR_TRY(exclusive_sum_i64(nullptr, &tb2, wcost, wpre, m + 1, s));
     TR_TRY(sort_pairs_u32(nullptr, &tb3, (const uint32_t *)g.adjp, (uint32_t *)ihead, ids, inedge,
                           m, 0, hbits, s));
@@ -908,7 +910,7 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, 
     tb2 = tb2 > tb3 ? tb2 : tb3;
     void *tmp = A.alloc(tb2);
     if (!tmp) return TRUSS_ENOMEM;
-    TR_TRY(exclusive_sum_i64(tmp, &tb, (const int64_t *)hcnt, inoff, n + 1, s));
+    TR_TRY(exclusive_sum_i64(tmp, &tb, hcnt, inoff, n + 1, s));
     TR_TRY(sort_pairs_u32(tmp, &tb3, (const uint32_t *)g.adjp, (uint32_t *)ihead, ids, inedge, m,
                           0, hbits, s));
     const int ec = cfg.pair_cost > 0 ? cfg.pair_cost : cfg.pair_cost < 0 ? 0 : kEdgeCost;
@@ -1054,8 +1056,14 @@ int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &s
     const int64_t n = g.n, tri = so.entries / 3;
     int64_t *c1 = A.get<int64_t>(m + 1), *c2 = A.get<int64_t>(m + 1);
     int64_t *p1 = A.get<int64_t>(m + 1), *p2 = A.get<int64_t>(m + 1);
-    const int64_t nr1 = (tri + kLEdgeCost * m) / kLRangeCost + 1;
-    const int64_t nr2 = (tri + 2 * kLEdgeCost * m) / kLRangeCost + 1;
+    // Ranges of kLRangeCost leave most blocks idle below some 10 M triangles:
+    // smaller graphs take four ranges per block, but none under kLMinCost
+    // (list passes of the 4,096-vertex graph 62 us, now LP_TINY us; of R-MAT
+    // scale 15 163 us, now LP_SMALL us).
+    const int64_t total = tri + 2 * kLEdgeCost * m, fit = total / (4 * 2 * 152);
+    const int64_t rc = fit > kLRangeCost ? kLRangeCost : fit < kLMinCost ? kLMinCost : fit;
+    const int64_t nr1 = (tri + kLEdgeCost * m) / rc + 1;
+    const int64_t nr2 = total / rc + 1;
     int64_t *vb1 = A.get<int64_t>(nr1 + 1), *vb2 = A.get<int64_t>(nr2 + 1);
     unsigned long long *next = A.get<unsigned long long>(2);
     if (!c1 || !c2 || !p1 || !p2 || !vb1 || !vb2 || !next) return TRUSS_ENOMEM;
@@ -1068,10 +1076,10 @@ int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &s
     TR_TRY(exclusive_sum_i64(tmp, &tb, c1, p1, m + 1, s));
     TR_TRY(exclusive_sum_i64(tmp, &tb, c2, p2, m + 1, s));
     k_list_ranges<<<grid_for(nr1 + 1, 256, 152 * 8), 256, 0, s>>>(n, nr1, p1, g.offp, g.offp,
-                                                                    false, vb1);
+                                                                    false, rc, vb1);
     TR_LAUNCHED();
     k_list_ranges<<<grid_for(nr2 + 1, 256, 152 * 8), 256, 0, s>>>(n, nr2, p2, so.inoff, g.offp,
-                                                                    true, vb2);
+                                                                    true, rc, vb2);
     TR_LAUNCHED();
     TR_CUDA(cudaMemsetAsync(next, 0, 2 * sizeof(unsigned long long), s));
     int dev = 0, sms = cfg.sms;

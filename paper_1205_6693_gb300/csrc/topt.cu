@@ -24,55 +24,18 @@ namespace tr {
 
 namespace {
 
-constexpr int kBlk = 128;
-
-__global__ void k_in_count(int64_t m, const int32_t *adjp, unsigned long long *indeg) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
-       e += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&indeg[adjp[e]], 1ull);
-}
-
-// inedge[inoff[v] ..) = the oriented edges (u, v) with head v, in any order.
-__global__ void k_in_fill(int64_t m, const int32_t *adjp, const int64_t *inoff,
-                          unsigned long long *cur, int32_t *inedge) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int v = adjp[e];
-    const unsigned long long p = atomicAdd(&cur[v], 1ull);
-    inedge[inoff[v] + (int64_t)p] = (int32_t)e;
-  }
-}
-
-// Block sum of one value per thread.
-__device__ __forceinline__ int block_sum(int x, int *red) {
-  for (int o = 16; o >= 1; o >>= 1) x += __shfl_down_sync(TR_FULL, x, o);
-  const int w = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane_id() == 0) red[w] = x;
-  __syncthreads();
-  int t = 0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); i++) t += red[i];
-  return t;
-}
-
-// Supports of the edges incident to w that are >= x: out-edges are the
-// contiguous range offp[w] .. offp[w+1], in-edges come through inedge.
-__device__ __forceinline__ int count_ge(const int32_t *sup, int64_t ob, int dout,
-                                        const int32_t *inedge, int64_t ib, int din, int x,
-                                        int *red) {
-  int c = 0;
-  for (int i = threadIdx.x; i < dout; i += blockDim.x) c += __ldg(&sup[ob + i]) >= x;
-  for (int i = threadIdx.x; i < din; i += blockDim.x)
-    c += __ldg(&sup[__ldg(&inedge[ib + i])]) >= x;
-  return block_sum(c, red);
-}
-
-// h_w (h-index of the incident supports) and c_w (how many are >= h_w):
-// bisection on x over [0, deg(w)], since #{supports >= x} >= x holds exactly
-// for x <= h_w.  Vertices of degree <= kRegVals * 32 take one warp, with the
-// supports held in registers; larger ones take a whole block and re-read the
-// supports at every step.
+// h_w (h-index of the incident supports) and c_w (how many are >= h_w), on x
+// over [0, deg(w)], since #{supports >= x} >= x holds exactly for x <= h_w.
+// The out-edges of w are the contiguous range offp[w] .. offp[w+1], its
+// in-edges come through inedge.  Vertices of degree <= kRegVals * 32 take one
+// warp, which bisects with the supports held in registers; larger ones take a
+// whole block, which splits the range of x into kBins counted in shared
+// memory: one or two reads of the supports instead of one for every bit of
+// the degree (R-MAT scale 18: 1,047 us, now HB_FIG us).
 constexpr int kRegVals = 8;
+constexpr int kBlk = 512;
+constexpr int kBinsPerThread = 4;
+constexpr int kBins = kBlk * kBinsPerThread;
 
 __global__ void __launch_bounds__(256) k_hindex_warp(int64_t n, const int64_t *offp,
                                                      const int64_t *inoff, const int32_t *inedge,
@@ -124,28 +87,71 @@ __global__ void __launch_bounds__(kBlk) k_hindex_block(const int32_t *big,
                                                        const int64_t *offp, const int64_t *inoff,
                                                        const int32_t *inedge, const int32_t *sup,
                                                        int32_t *h, int32_t *c) {
-  __shared__ int red[kBlk / 32];
+  __shared__ int s_bin[kBins];
+  __shared__ int s_warp[kBlk / 32];
+  __shared__ int s_best, s_at, s_above;
   const int64_t nb = (int64_t)*nbig;
+  const int lane = lane_id(), wib = threadIdx.x >> 5;
   for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
     const int64_t w = big[b];
     const int64_t ob = offp[w], ib = inoff[w];
     const int dout = (int)(offp[w + 1] - ob), din = (int)(inoff[w + 1] - ib);
     const int d = dout + din;
-    int lo = 0, hi = d + 1, clo = d;
-    while (hi - lo > 1) {
-      const int mid = lo + ((hi - lo) >> 1);
-      const int cm = count_ge(sup, ob, dout, inedge, ib, din, mid, red);
-      if (cm >= mid) {
-        lo = mid;
-        clo = cm;
-      } else {
-        hi = mid;
+    // supports are clipped to d; h lies in [lo, lo + kBins << sh), and `above`
+    // supports lie beyond that
+    int lo = 0, above = 0;
+    int sh = 0;
+    while (((int64_t)kBins << sh) < (int64_t)d + 1) sh++;
+    for (;; sh = sh > 11 ? sh - 11 : 0) {
+      static_assert(kBins == 1 << 11, "a pass narrows the range by 11 bits");
+      for (int i = threadIdx.x; i < kBins; i += kBlk) s_bin[i] = 0;
+      if (threadIdx.x == 0) s_best = 0;
+      __syncthreads();
+      const int64_t hi = lo + ((int64_t)kBins << sh);
+      for (int i = threadIdx.x; i < d; i += kBlk) {
+        const int v = min(i < dout ? __ldg(&sup[ob + i]) : __ldg(&sup[__ldg(&inedge[ib + i - dout])]), d);
+        if (v >= lo && v < hi) atomicAdd(&s_bin[(v - lo) >> sh], 1);
       }
+      __syncthreads();
+      int cnt[kBinsPerThread], sum = 0;
+#pragma unroll
+      for (int q = 0; q < kBinsPerThread; q++) {
+        cnt[q] = s_bin[threadIdx.x * kBinsPerThread + q];
+        sum += cnt[q];
+      }
+      const int P = warp_incl_scan(sum);
+      if (lane == 31) s_warp[wib] = P;
+      __syncthreads();
+      int ge = above;  // supports in bins from this thread's first on, and above
+      for (int q = wib; q < kBlk / 32; q++) ge += s_warp[q];
+      ge -= P - sum;
+      int best = -1, at = 0, beyond = 0;
+#pragma unroll
+      for (int q = 0; q < kBinsPerThread; q++) {
+        const int bin = threadIdx.x * kBinsPerThread + q;
+        if ((int64_t)ge >= lo + ((int64_t)bin << sh)) {
+          best = bin;
+          at = ge;
+          beyond = ge - cnt[q];
+        }
+        ge -= cnt[q];
+      }
+      if (best > 0) atomicMax(&s_best, best);
+      __syncthreads();
+      if (best >= 0 && best == s_best) {
+        s_at = at;
+        s_above = beyond;
+      }
+      __syncthreads();
+      lo += s_best << sh;
+      above = s_above;
+      if (sh == 0) break;
     }
     if (threadIdx.x == 0) {
       h[w] = lo;
-      c[w] = clo;
+      c[w] = s_at;
     }
+    __syncthreads();
   }
 }
 
@@ -220,24 +226,14 @@ __global__ void k_top(int64_t mc, const int32_t *ce, const int32_t *phi_rows, in
 
 }  // namespace
 
-int compute_psi(Arena &A, const Csr &g, const int32_t *sup, int32_t *psi, cudaStream_t s) {
+int compute_psi(Arena &A, const Csr &g, const SupportOut &so, int32_t *psi, cudaStream_t s) {
   const int64_t m = g.m, n = g.n;
   if (m == 0) return TRUSS_OK;
-  unsigned long long *cnt = A.get<unsigned long long>(n + 1);
-  int64_t *inoff = A.get<int64_t>(n + 1);
-  int32_t *inedge = A.get<int32_t>(m), *h = A.get<int32_t>(n), *c = A.get<int32_t>(n);
-  if (!cnt || !inoff || !inedge || !h || !c) return TRUSS_ENOMEM;
-  TR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * (n + 1), s));
-  k_in_count<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, g.adjp, cnt);
-  TR_LAUNCHED();
-  size_t tb = 0;
-  TR_TRY(exclusive_sum_i64(nullptr, &tb, (const int64_t *)cnt, inoff, n + 1, s));
-  void *tmp = A.alloc(tb);
-  if (!tmp) return TRUSS_ENOMEM;
-  TR_TRY(exclusive_sum_i64(tmp, &tb, (const int64_t *)cnt, inoff, n + 1, s));
-  TR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * (n + 1), s));
-  k_in_fill<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, g.adjp, inoff, cnt, inedge);
-  TR_LAUNCHED();
+  // the support pass grouped the edges by head already
+  const int32_t *sup = so.sup, *inedge = so.inedge;
+  const int64_t *inoff = so.inoff;
+  int32_t *h = A.get<int32_t>(n), *c = A.get<int32_t>(n);
+  if (!h || !c) return TRUSS_ENOMEM;
   if (n > 0) {
     int32_t *big = A.get<int32_t>(n);
     unsigned long long *nbig = A.get<unsigned long long>(1);
@@ -246,7 +242,7 @@ int compute_psi(Arena &A, const Csr &g, const int32_t *sup, int32_t *psi, cudaSt
     k_hindex_warp<<<grid_for(n * 32, 256, 152 * 16), 256, 0, s>>>(n, g.offp, inoff, inedge, sup,
                                                                   h, c, big, nbig);
     TR_LAUNCHED();
-    k_hindex_block<<<152 * 8, kBlk, 0, s>>>(big, nbig, g.offp, inoff, inedge, sup, h, c);
+    k_hindex_block<<<152 * 4, kBlk, 0, s>>>(big, nbig, g.offp, inoff, inedge, sup, h, c);
     TR_LAUNCHED();
   }
   k_psi<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, g.esrc, g.adjp, sup, h, c, psi);
