@@ -84,6 +84,16 @@ size_t Arena::headroom(size_t free_dev) const {
   return left < room ? left : room;
 }
 
+bool Arena::has_room(double bytes) const {
+  if (bytes < (double)headroom(0)) return true;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    fr = 0;
+  }
+  return bytes < (double)headroom(fr);
+}
+
 size_t Arena::unused() const {
   size_t s = 0;
   for (auto &c : chunks_) s += c.cap - c.used;
@@ -393,11 +403,6 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
   }
   TR_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), s));
 
-  tr::Csr g;
-  TR_TRY(tr::build_csr(A, in, &g, ctx->d_err, s));
-  sg.mark();  // 1
-  st.m = g.m;
-
   tr::SupportCfg scfg;
   scfg.sms = ctx->sms;
   scfg.records = want_truss && !ctx->opts.lists_by_walk;
@@ -406,8 +411,14 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
   scfg.pair_cost = ctx->opts.support_pair_cost;
   scfg.range_work = ctx->opts.support_range_work;
   scfg.stage_max = ctx->opts.support_stage_max;
+  scfg.small_paths = ctx->opts.wait_limit_ns <= 0;
+  tr::Csr g;
+  tr::SupportPrep prep;
+  TR_TRY(tr::build_graph(A, in, scfg, &g, &prep, ctx->d_err, s));
+  sg.mark();  // 1
+  st.m = g.m;
   tr::SupportOut so;
-  TR_TRY(tr::run_support(A, g, scfg, &so, s));
+  TR_TRY(tr::run_support(A, g, scfg, prep, &so, s));
   sg.mark();  // 2
   st.triangles = so.entries / 3;
   if (graph_m && h_row_off) {
@@ -427,6 +438,27 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
 
   int32_t *truss_e = nullptr;
   tr::PeelResult pr;
+  // the per-row outputs, enqueued behind the kernels that compute them; they
+  // are written once, by the scatter: pinned host outputs in place
+  auto emit = [&]() -> int {
+    sg.mark();  // 4 (or 3 for support only: the scatter ends at the next)
+    OutBuf os, ot;
+    TR_TRY(stage_out(A, support_out, rows, &os, true));
+    TR_TRY(stage_out(A, want_truss ? truss_out : nullptr, rows, &ot, true));
+    TR_TRY(tr::scatter_rows_packed(A, g, so.sup, truss_e, os.dev, ot.dev, s));
+    if (G > 1 || h_row_off) {
+      if (kmax_out && want_truss) {
+        OutBuf ok;
+        TR_TRY(stage_out(A, kmax_out, G, &ok));
+        TR_TRY(tr::batch_kmax(G, d_row_off, ot.dev, ok.dev, s));
+        TR_TRY(copy_back(ok, G, s));
+      }
+    }
+    TR_TRY(copy_back(os, rows, s));
+    TR_TRY(copy_back(ot, rows, s));
+    sg.mark();  // 5
+    return TRUSS_OK;
+  };
   if (want_truss) {
     // peel variant 4: the barrier-free peel, which needs the full lists and
     // a triangle id per list entry (record indices, so records and fewer
@@ -447,35 +479,19 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
     pcfg.variant = ctx->opts.peel_variant;
     pcfg.count = ctx->opts.count_bytes != 0 && !tids;
     if (ctx->opts.wait_limit_ns > 0) pcfg.wait_ns = ctx->opts.wait_limit_ns;
+    pcfg.then = emit;
     int rc = tids ? tr::run_peel_async(A, g, so, pairs, tids, so.records, pcfg, truss_e, &pr, s)
                   : tr::run_peel(A, g, so, lists, pcfg, truss_e, &pr, s);
     if (rc != TRUSS_OK) return rc;
-    sg.mark();  // 4
     st.kmax = pr.kmax;
     st.levels = pr.levels;
     st.subrounds = pr.subrounds;
     st.peel_entries = (int64_t)pr.entries;
     st.peel_decrements = (int64_t)pr.decrements;
     st.peel_scanned = (int64_t)pr.scanned;
+  } else {
+    TR_TRY(emit());
   }
-
-  // the per-row outputs are written once, by the scatter: pinned host
-  // outputs in place
-  OutBuf os, ot;
-  TR_TRY(stage_out(A, support_out, rows, &os, true));
-  TR_TRY(stage_out(A, want_truss ? truss_out : nullptr, rows, &ot, true));
-  TR_TRY(tr::scatter_rows_packed(A, g, so.sup, truss_e, os.dev, ot.dev, s));
-  if (G > 1 || h_row_off) {
-    if (kmax_out && want_truss) {
-      OutBuf ok;
-      TR_TRY(stage_out(A, kmax_out, G, &ok));
-      TR_TRY(tr::batch_kmax(G, d_row_off, ot.dev, ok.dev, s));
-      TR_TRY(copy_back(ok, G, s));
-    }
-  }
-  TR_TRY(copy_back(os, rows, s));
-  TR_TRY(copy_back(ot, rows, s));
-  sg.mark();  // 5 (or 3 for support only)
   int32_t k_host = pr.kmax;
   if (!(G > 1 || h_row_off) && kmax_out && want_truss) {
     if (is_device_ptr(kmax_out)) {
@@ -494,8 +510,8 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
       st.ms_scatter = sg.ms(4, 5);
       st.ms_total = sg.ms(0, 5);
     } else {
-      st.ms_scatter = sg.ms(2, 3);
-      st.ms_total = sg.ms(0, 3);
+      st.ms_scatter = sg.ms(3, 4);
+      st.ms_total = sg.ms(0, 4);
     }
   }
   st.launches = tr::take_launches();
@@ -544,8 +560,6 @@ int decompose_device_rows(truss_ctx *ctx, tr::Arena &A, const tr::RowsIn &in, in
                           tr::PeelResult *pr, cudaStream_t s) {
   *pr = tr::PeelResult{};
   if (in.rows == 0) return TRUSS_OK;
-  tr::Csr g;
-  TR_TRY(tr::build_csr(A, in, &g, ctx->d_err, s));
   tr::SupportCfg cfg;
   cfg.sms = ctx->sms;
   cfg.records = true;
@@ -553,8 +567,12 @@ int decompose_device_rows(truss_ctx *ctx, tr::Arena &A, const tr::RowsIn &in, in
   cfg.pair_cost = ctx->opts.support_pair_cost;
   cfg.range_work = ctx->opts.support_range_work;
   cfg.stage_max = ctx->opts.support_stage_max;
+  cfg.small_paths = ctx->opts.wait_limit_ns <= 0;
+  tr::Csr g;
+  tr::SupportPrep prep;
+  TR_TRY(tr::build_graph(A, in, cfg, &g, &prep, ctx->d_err, s));
   tr::SupportOut so;
-  TR_TRY(tr::run_support(A, g, cfg, &so, s));
+  TR_TRY(tr::run_support(A, g, cfg, prep, &so, s));
   int2 *pairs = A.get<int2>(tr::list_rest_entries(so));
   int32_t *truss_e = A.get<int32_t>(g.m);
   if (!pairs || !truss_e) return TRUSS_ENOMEM;
@@ -571,9 +589,8 @@ int decompose_device_rows(truss_ctx *ctx, tr::Arena &A, const tr::RowsIn &in, in
     TR_TRY(tr::pin_edges(g.rows, g.row2e, pinned_rows, pe, g.m, s));
     pcfg.pinned = pe;
   }
-  int rc = tr::run_peel(A, g, so, lists, pcfg, truss_e, pr, s);
-  if (rc != TRUSS_OK) return rc;
-  return tr::scatter_rows(g, so.sup, truss_e, sup_rows, truss_rows, s);
+  pcfg.then = [&]() { return tr::scatter_rows(g, so.sup, truss_e, sup_rows, truss_rows, s); };
+  return tr::run_peel(A, g, so, lists, pcfg, truss_e, pr, s);
 }
 
 // Per-row support and psi (Procedure 6) of the graph the rows define.
@@ -593,16 +610,18 @@ int run_upper_bound(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src,
   TR_TRY(stage_in(A, src, rows, &in.src, s));
   TR_TRY(stage_in(A, dst, rows, &in.dst, s));
   TR_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), s));
-  tr::Csr g;
-  TR_TRY(tr::build_csr(A, in, &g, ctx->d_err, s));
-  st.m = g.m;
   tr::SupportCfg scfg;
   scfg.sms = ctx->sms;
+  scfg.small_paths = ctx->opts.wait_limit_ns <= 0;
   scfg.pair_cost = ctx->opts.support_pair_cost;
   scfg.range_work = ctx->opts.support_range_work;
   scfg.stage_max = ctx->opts.support_stage_max;
+  tr::Csr g;
+  tr::SupportPrep prep;
+  TR_TRY(tr::build_graph(A, in, scfg, &g, &prep, ctx->d_err, s));
+  st.m = g.m;
   tr::SupportOut so;
-  TR_TRY(tr::run_support(A, g, scfg, &so, s));
+  TR_TRY(tr::run_support(A, g, scfg, prep, &so, s));
   st.triangles = so.entries / 3;
   int32_t *psi = A.get<int32_t>(g.m);
   if (!psi) return TRUSS_ENOMEM;
@@ -648,16 +667,18 @@ int run_top(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src, const i
   TR_TRY(stage_in(A, src, rows, &in.src, s));
   TR_TRY(stage_in(A, dst, rows, &in.dst, s));
   TR_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), s));
-  tr::Csr g;
-  TR_TRY(tr::build_csr(A, in, &g, ctx->d_err, s));
-  st.m = g.m;
   tr::SupportCfg scfg;
   scfg.sms = ctx->sms;
+  scfg.small_paths = ctx->opts.wait_limit_ns <= 0;
   scfg.pair_cost = ctx->opts.support_pair_cost;
   scfg.range_work = ctx->opts.support_range_work;
   scfg.stage_max = ctx->opts.support_stage_max;
+  tr::Csr g;
+  tr::SupportPrep prep;
+  TR_TRY(tr::build_graph(A, in, scfg, &g, &prep, ctx->d_err, s));
+  st.m = g.m;
   tr::SupportOut so;
-  TR_TRY(tr::run_support(A, g, scfg, &so, s));
+  TR_TRY(tr::run_support(A, g, scfg, prep, &so, s));
   st.triangles = so.entries / 3;
   int32_t *psi = A.get<int32_t>(g.m), *top = A.get<int32_t>(g.m);
   int32_t *cs = A.get<int32_t>(g.m), *cd = A.get<int32_t>(g.m), *ce = A.get<int32_t>(g.m);
@@ -792,19 +813,21 @@ int run_bottom_up(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src,
   TR_TRY(stage_in(A, src, rows, &in.src, s));
   TR_TRY(stage_in(A, dst, rows, &in.dst, s));
   TR_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), s));
-  tr::Csr g;
-  TR_TRY(tr::build_csr(A, in, &g, ctx->d_err, s));
-  const int64_t m = g.m;
-  st.m = m;
   // supports of the whole graph: the support pass needs no triangle lists,
   // so its working set is a few words per edge
   tr::SupportCfg scfg;
   scfg.sms = ctx->sms;
+  scfg.small_paths = ctx->opts.wait_limit_ns <= 0;
   scfg.pair_cost = ctx->opts.support_pair_cost;
   scfg.range_work = ctx->opts.support_range_work;
   scfg.stage_max = ctx->opts.support_stage_max;
+  tr::Csr g;
+  tr::SupportPrep prep;
+  TR_TRY(tr::build_graph(A, in, scfg, &g, &prep, ctx->d_err, s));
+  const int64_t m = g.m;
+  st.m = m;
   tr::SupportOut so;
-  TR_TRY(tr::run_support(A, g, scfg, &so, s));
+  TR_TRY(tr::run_support(A, g, scfg, prep, &so, s));
   st.triangles = so.entries / 3;
   const int32_t *supx = so.sup;
   int32_t *lower = A.get<int32_t>(m), *phi = A.get<int32_t>(m);

@@ -174,6 +174,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long *bar, int *err,
   return s_ok != 0;
 }
 
+// r W / P without overflowing 64 bits (r <= P <= m).
+__device__ __forceinline__ int64_t range_point(int64_t W, int64_t P, int64_t r) {
+  return (W / P) * r + (W % P) * r / P;
+}
+
 // ----------------------------------------------- phases of a persistent peel ---
 // What a scan found (slot = scan index % 3).
 struct __align__(16) ScanOut {

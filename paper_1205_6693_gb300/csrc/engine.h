@@ -3,6 +3,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -43,6 +44,9 @@ class Arena {
   // memory: what the cap leaves, and no more than the reserved chunks' spare
   // room plus free_dev.
   size_t headroom(size_t free_dev) const;
+  // Whether that is more than `bytes`; asks the device for its free memory
+  // only if the reserved chunks alone do not settle it.
+  bool has_room(double bytes) const;
   void release_all();
   // Allocation state, to hand back everything allocated after it (rewind);
   // chunks reserved since stay reserved.
@@ -89,6 +93,15 @@ struct RowsIn {
   const int64_t *voff = nullptr;
 };
 
+// Small control words of one decomposition, zeroed together by build_graph:
+// one memset instead of one per kernel that needs a cleared counter.
+struct ZeroBlock {
+  static constexpr size_t kCtl = 512;
+  alignas(16) unsigned char build[kCtl], offsets[kCtl], peel[kCtl];
+  unsigned long long list_next[2];
+  int list_err;  // set by the list builders, reported with the peel's result
+};
+
 // Degree-ordered oriented CSR (vertices relabelled by ascending (degree, id)
 // so that an edge points from its lower-ranked to its higher-ranked end).
 // Canonical edge id e = position in adjp.
@@ -100,6 +113,7 @@ struct Csr {
   int32_t *row2e = nullptr;  // [rows] row -> e, -1 for self-loop rows
   int32_t *order = nullptr;  // [n]   rank -> input vertex id
   int32_t *sdeg = nullptr;   // [n]   degree of the vertex of each rank (ascending)
+  ZeroBlock *zero = nullptr; // set by build_graph
 };
 
 struct DevCounters;  // device scratch for small counters (api.cu)
@@ -107,6 +121,12 @@ struct DevCounters;  // device scratch for small counters (api.cu)
 int build_csr(Arena &A, const RowsIn &in, Csr *out, int32_t *d_err, cudaStream_t s);
 
 // ------------------------------------------------------------- support ---
+// What the passes over whole lists need of a small graph: cursors, cost
+// prefixes and vertex ranges (small.cu).
+struct SmallLists {
+  unsigned long long *cur = nullptr;
+  int64_t *p1 = nullptr, *p2 = nullptr, *vb1 = nullptr, *vb2 = nullptr;
+};
 struct SupportOut {
   int32_t *sup = nullptr;    // [m]  sup(e)
   int32_t *supA = nullptr;   // [m]  triangles in which e is e_uv or e_uw (e in out(u))
@@ -121,6 +141,35 @@ struct SupportOut {
   int2 *tb = nullptr;        // (e_uw, e_vw) records per walked edge e_uv
   int32_t *cuv = nullptr;    // [m] records per edge
   bool in_place = false;     // the lists keep each edge's own part in its records
+  SmallLists small;          // small graphs: ready for the passes over whole lists
+};
+
+// Cost of one vertex range of the list passes (support.cu), and how many
+// ranges the two passes take.
+struct ListRanges {
+  int64_t cost, n1, n2;
+};
+constexpr int kListEdgeCost = 4;  // range cost per edge (next to its records)
+constexpr int kListCounters = 16384;  // shared cursor counters per range (64 KB)
+__host__ __device__ inline ListRanges list_ranges(int64_t triangles, int64_t m) {
+  // A range's out-edges should fit the counters.  Ranges of that size leave
+  // most blocks idle on small graphs: those take four ranges per block, but
+  // none under kMin (list passes of the 4,096-vertex graph 62 -> 25 us; of
+  // R-MAT scale 15 the same 165 us).
+  constexpr int64_t kMax = (int64_t)kListCounters * kListEdgeCost / 2, kMin = 512;
+  const int64_t total = triangles + 2 * kListEdgeCost * m, fit = total / (4 * 2 * 152);
+  const int64_t cost = fit > kMax ? kMax : fit < kMin ? kMin : fit;
+  return {cost, (triangles + kListEdgeCost * m) / cost + 1, total / cost + 1};
+}
+
+// What a small graph's build leaves ready for the support walk (small.cu).
+struct SupportPrep {
+  bool valid = false;
+  int32_t *supA = nullptr, *supB = nullptr;  // [m] zeroed
+  int32_t *cuv = nullptr;                    // [m] zeroed (null: not prepared)
+  int32_t *inedge = nullptr, *ihead = nullptr;
+  int64_t *inoff = nullptr, *wcost = nullptr, *wpre = nullptr, *tbpre = nullptr, *rb = nullptr;
+  int64_t W = 0, R = 0, P = 0;
 };
 
 struct SupportCfg {
@@ -132,10 +181,29 @@ struct SupportCfg {
   int pair_cost = 0;      // fixed cost per oriented edge, in out-list entries (0 = default, <0 = none)
   int64_t range_work = 0; // walk cost per range (0 = default)
   int stage_max = 0;      // stage out-lists of at most this many entries (0 = capacity)
+  // small graphs may take the paths of small.cu, whose launches wait at grid
+  // barriers (not for a caller that bounds its waits: those paths would have
+  // to fail where the general ones do not wait)
+  bool small_paths = false;
 };
 
+// CSR build: the path for small graphs when the configuration allows it and
+// the sizes suit it (then *prep is valid), else build_csr.
+int build_graph(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, SupportPrep *prep,
+                int32_t *d_err, cudaStream_t s);
+// Per-edge costs and default of the walk's ranges, resident warps of the walk.
+int walk_edge_cost(const SupportCfg &cfg);
+int64_t walk_range_work(const SupportCfg &cfg);
+int walk_warps(const SupportCfg &cfg, int64_t *warps);
+
+// Supports, list offsets and what the list passes need, of a small graph whose
+// walk has run (small.cu): sup, toff [m+1]; with records (cuv) also *lists.
+int small_offsets(Arena &A, const Csr &g, const SupportPrep &prep, const int32_t *cuv, int sms,
+                  int32_t *sup, int64_t *toff, int64_t *total, SmallLists *lists, cudaStream_t s);
+
 // Support of every edge: sup = supA + supB (support.cu).
-int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, cudaStream_t s);
+int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportPrep &prep,
+                SupportOut *out, cudaStream_t s);
 // Where the triangle list of each edge lives: for edge e, the other two
 // edge ids of each triangle of e are own[own_off[e] .. own_off[e] +
 // own_cnt[e]) followed by rest[off[e] .. off[e] + sup[e] - own_cnt[e]).
@@ -161,6 +229,7 @@ inline int64_t list_rest_entries(const SupportOut &so) {
 // Triangle lists (support.cu) into `pairs` (list_rest_entries entries).
 // tids (nullable, only with records and whole lists): the record index of
 // each entry's triangle, for the barrier-free peel.
+// A list that would overflow sets g.zero->list_err, which the peel reports.
 int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &so, int2 *pairs,
               uint32_t *tids, TriLists *out, cudaStream_t s);
 
@@ -175,6 +244,9 @@ struct PeelCfg {
   // last level to run (0 = all).  Edges not removed by then get truss 0.
   const uint8_t *pinned = nullptr;
   int k_stop = 0;
+  // Called once the peel is enqueued, before its result is read back: work
+  // that needs only the device's truss numbers (no gap before it on the GPU).
+  std::function<int()> then;
   // Counting run (untimed): record each edge's removal sub-round and the
   // per-level list-entry counts, and compute the algorithmic bytes of the
   // removals (PeelResult::sum_min_alive .. alive_levels).

@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
 constexpr int kPinnedRes = INT_MAX / 4;
 
 __global__ void k_peel_init(int64_t m, const int32_t *sup, const uint8_t *pinned, uint32_t *word,
-                            int32_t *alive, int32_t *truss, PeelCtl *ctl) {
+                            int32_t *alive, int32_t *truss, const int *list_err, PeelCtl *ctl) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
     word[e] = (uint32_t)((pinned && pinned[e]) ? kPinnedRes : sup[e]);
@@ -702,6 +702,7 @@ __global__ void k_peel_init(int64_t m, const int32_t *sup, const uint8_t *pinned
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     for (int i = 0; i < 3; i++) ctl->scan[i].minres = INT_MAX;
+    ctl->err = *list_err;  // a list builder's error is reported with the peel's result
   }
 }
 
@@ -852,7 +853,7 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
              int32_t *truss, PeelResult *out, cudaStream_t s) {
   const int64_t m = g.m;
   *out = PeelResult{};
-  if (m == 0) return TRUSS_OK;
+  if (m == 0) return cfg.then ? cfg.then() : TRUSS_OK;
   // items carry 32-bit block numbers
   if (so.entries >= kOffLimit || (L.own_cnt && so.records >= kOffLimit)) return TRUSS_EINVAL;
   if (so.entries > 0 && (!L.rest || !L.off || (L.own_cnt && (!L.own || !L.own_off))))
@@ -868,11 +869,11 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
   uint32_t *word = A.get<uint32_t>(m);
   int32_t *al0 = A.get<int32_t>(m), *al1 = A.get<int32_t>(m);
   int4 *Q = A.get<int4>(item_cap);
-  PeelCtl *ctl = A.get<PeelCtl>(1);
-  if (!word || !al0 || !al1 || !Q || !ctl) return TRUSS_ENOMEM;
-  TR_CUDA(cudaMemsetAsync(ctl, 0, sizeof(PeelCtl), s));
+  static_assert(sizeof(PeelCtl) <= ZeroBlock::kCtl, "control words fit the zero block");
+  PeelCtl *ctl = (PeelCtl *)g.zero->peel;
+  if (!word || !al0 || !al1 || !Q) return TRUSS_ENOMEM;
   k_peel_init<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, so.sup, cfg.pinned, word, al0, truss,
-                                                          ctl);
+                                                          &g.zero->list_err, ctl);
   TR_LAUNCHED();
 
   int dev = 0, sms = cfg.sms;
@@ -947,6 +948,7 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
   void *args[] = {&a};
   TR_CUDA(cudaLaunchCooperativeKernel(kern, dim3(sms * occ), dim3(kPeelBlock), args, 0, s));
   count_launches(1);
+  if (cfg.then) TR_TRY(cfg.then());
   PeelCtl h{};
   TR_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(PeelCtl), cudaMemcpyDeviceToHost, s));
   TR_CUDA(cudaStreamSynchronize(s));

@@ -381,7 +381,7 @@ int run_peel_async(Arena &A, const Csr &g, const SupportOut &so, const int2 *pai
                    PeelResult *out, cudaStream_t s) {
   const int64_t m = g.m;
   *out = PeelResult{};
-  if (m == 0) return TRUSS_OK;
+  if (m == 0) return cfg.then ? cfg.then() : TRUSS_OK;
   // every edge is queued once: at most max(1, ceil(sup / kItem)) items each
   const int64_t item_cap = m + so.entries / kItem + 64;
   const int64_t words = (ntri + 31) / 32 + 1;
@@ -425,9 +425,13 @@ int run_peel_async(Arena &A, const Csr &g, const SupportOut &so, const int2 *pai
   TR_CUDA(cudaLaunchCooperativeKernel((const void *)k_peel_async, dim3(sms * occ), dim3(kBlock),
                                       args, 0, s));
   count_launches(1);
+  if (cfg.then) TR_TRY(cfg.then());
   AsyncCtl h{};
+  int list_err = 0;
+  TR_CUDA(cudaMemcpyAsync(&list_err, &g.zero->list_err, sizeof(int), cudaMemcpyDeviceToHost, s));
   TR_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(AsyncCtl), cudaMemcpyDeviceToHost, s));
   TR_CUDA(cudaStreamSynchronize(s));
+  if (h.err == 0 && list_err != 0) h.err = TRUSS_ECHECK;
   out->err = h.err;
   out->kmax = h.kmax;
   out->levels = h.levels;

@@ -32,8 +32,14 @@ constexpr int kEdgeCost = 64;          // fixed walk cost per oriented edge (ent
 // its counts (int32) and a position table of kHashSlots uint16 slots.
 constexpr int kHeadCap = 512;
 // Out-lists shorter than this are not staged: their few probes go to the
-// L1-cached global list (batch of small graphs: support 11.1 -> 10.3 ms).
-constexpr int kStageMin = 16;
+// L1-cached global list, and their in-edges are walked 32 at a time whichever
+// heads they belong to (one head at a time paid a chain of some ten dependent
+// loads per head).  Support stage with lists under 16 one head at a time / with
+// mixed walks under 16 / 32 / 64: 4,096 small graphs 7.21 / 4.69 / 4.65 / 4.78
+// ms, 10 M Chung-Lu rows 2.46 / 2.23 / 2.21 / 2.24, 2.1 M random rows 0.61 /
+// 0.22 / 0.23 / 0.24, R-MAT scale 20 9.37 / 9.39 / 9.44 / 9.55.
+constexpr int kStageMin = 32;
+constexpr int kMixedMax = 32;  // a power of two, at least kStageMin
 constexpr int kHashSlots = 2048;
 constexpr size_t kHeadSmem = (size_t)kHeadCap * 8 + (size_t)kHashSlots * 2;
 // List walk (the list builder used when the triangle records do not fit):
@@ -60,11 +66,6 @@ struct ListArgs {
   int64_t entries;      // size of pairs (writes beyond it are dropped)
   int *err;             // set to TRUSS_ECHECK if a list would overflow
 };
-
-// r W / P without overflowing 64 bits (r <= P <= m).
-__device__ __forceinline__ int64_t range_point(int64_t W, int64_t P, int64_t r) {
-  return (W / P) * r + (W % P) * r / P;
-}
 
 // First e in [0, m] with wpre[e] >= x.
 __device__ __forceinline__ int64_t lower_bound64(const int64_t *a, int64_t m, int64_t x) {
@@ -381,6 +382,104 @@ __device__ __forceinline__ void head_walk(const SupVArgs &a, int64_t i0, int64_t
   }
 }
 
+// Up to 32 in-edges (lane < cnt holds inedge[i0 + lane]) of heads with short
+// out-lists, whichever heads they are: lane o's head has the out-list
+// adjp[bv .. bv + dv), searched where it lies.  The walks are spread over the
+// lanes as in head_walk, so the warp pays the chain of dependent loads once
+// for 32 in-edges, not once for every head.
+__device__ __forceinline__ void mixed_walk(const SupVArgs &a, int64_t i0, int cnt, int bv, int dv) {
+  const int lane = lane_id();
+  const unsigned lt = (1u << lane) - 1u;
+  const bool valid = lane < cnt && dv > 0;
+  const int e = lane < cnt ? __ldg(&a.inedge[i0 + lane]) : 0;
+  const int len = valid ? (int)(__ldg(&a.wcost[i0 + lane]) - a.ecost) : 0;
+  const int64_t rb = (valid && a.tb) ? __ldg(&a.tbpre[e]) : 0;
+  const int vmax = valid ? __ldg(&a.adjp[bv + dv - 1]) : -1;
+  auto find = [&](int w, int b, int d) {
+    int q = 0;
+#pragma unroll
+    for (int step = kMixedMax / 2; step > 0; step >>= 1) {
+      const int nq = q + step;
+      if (nq <= d && __ldg(&a.adjp[b + nq - 1]) < w) q = nq;
+    }
+    return q < d && __ldg(&a.adjp[b + q]) == w ? q : -1;
+  };
+  const bool shrt = len <= kShortWalk;
+  const int sl = shrt ? len : 0;
+  const int P = warp_incl_scan(sl);
+  const int total = __shfl_sync(TR_FULL, P, 31);
+  int mycnt = 0;  // triangles found so far for this lane's (short) edge
+  for (int t0 = 0; t0 < total; t0 += 32 * kFlatU) {
+    int w[kFlatU], own[kFlatU], bo[kFlatU];
+#pragma unroll
+    for (int k = 0; k < kFlatU; k++) {
+      const int t = t0 + k * 32 + lane;
+      const bool act = t < total;
+      own[k] = warp_owner(P, act ? t : total - 1);
+      bo[k] = __shfl_sync(TR_FULL, P - sl, own[k]);
+      const int eo = __shfl_sync(TR_FULL, e, own[k]);
+      w[k] = act ? __ldg(&a.adjp[(int64_t)eo + 1 + (t - bo[k])]) : INT_MAX;
+    }
+#pragma unroll
+    for (int k = 0; k < kFlatU; k++) {
+      const int tr = t0 + k * 32;  // step of lane 0 in this round
+      if (tr >= total) break;
+      const int ob = __shfl_sync(TR_FULL, bv, own[k]), od = __shfl_sync(TR_FULL, dv, own[k]);
+      const int om = __shfl_sync(TR_FULL, vmax, own[k]);
+      const int q = w[k] <= om ? find(w[k], ob, od) : -1;
+      const unsigned hm = __ballot_sync(TR_FULL, q >= 0);
+      if (hm == 0) continue;
+      const int prior = __shfl_sync(TR_FULL, mycnt, own[k]);
+      const int64_t tbase = __shfl_sync(TR_FULL, rb, own[k]);
+      const int eo = __shfl_sync(TR_FULL, e, own[k]);
+      if (q >= 0) {
+        const int lo = max(bo[k] - tr, 0);
+        const unsigned below = hm & lt & ~((1u << lo) - 1u);
+        const int64_t euw = (int64_t)eo + 1 + (tr + lane - bo[k]);
+        count_hit<kSearch>(a, nullptr, ob, q, euw, tbase + prior + __popc(below));
+      }
+      if (sl > 0) {
+        const int lo = P - sl - tr, hi = P - 1 - tr;
+        if (hi >= 0 && lo <= 31) {
+          const int l0 = max(lo, 0), l1 = min(hi, 31);
+          const unsigned seg = (l1 == 31 ? 0xFFFFFFFFu : ((1u << (l1 + 1)) - 1u)) &
+                               ~((1u << l0) - 1u);
+          mycnt += __popc(hm & seg);
+        }
+      }
+    }
+  }
+  if (valid && shrt) {
+    if (a.tb) a.cuv[e] = mycnt;
+    if (mycnt) atomicAdd(&a.supA[e], mycnt);
+  }
+  // long walks: the whole warp on one edge, stopping past its head's max
+  unsigned lm = __ballot_sync(TR_FULL, valid && !shrt);
+  while (lm) {
+    const int o = __ffs(lm) - 1;
+    lm &= lm - 1;
+    const int eo = __shfl_sync(TR_FULL, e, o), olen = __shfl_sync(TR_FULL, len, o);
+    const int64_t tbase = __shfl_sync(TR_FULL, rb, o);
+    const int ob = __shfl_sync(TR_FULL, bv, o), od = __shfl_sync(TR_FULL, dv, o);
+    const int om = __shfl_sync(TR_FULL, vmax, o);
+    const int64_t start = (int64_t)eo + 1;
+    int c = 0;  // triangles of edge eo so far (warp-uniform)
+    for (int t0 = 0; t0 < olen; t0 += 32) {
+      const int t = t0 + lane;
+      const int w = t < olen ? __ldg(&a.adjp[start + t]) : INT_MAX;
+      const int q = w <= om ? find(w, ob, od) : -1;
+      const unsigned hm = __ballot_sync(TR_FULL, q >= 0);
+      if (q >= 0) count_hit<kSearch>(a, nullptr, ob, q, start + t, tbase + c + __popc(hm & lt));
+      c += __popc(hm);
+      if (__shfl_sync(TR_FULL, w, 31) > om) break;
+    }
+    if (lane == 0) {
+      if (a.tb) a.cuv[eo] = c;
+      if (c) atomicAdd(&a.supA[eo], c);
+    }
+  }
+}
+
 // Warps take equal-cost ranges of inedge round-robin; within a range, each
 // head's group is one segment with out(v) staged once.
 __global__ void __launch_bounds__(kBlock, 3) k_support_v(SupVArgs a) {
@@ -396,21 +495,30 @@ __global__ void __launch_bounds__(kBlock, 3) k_support_v(SupVArgs a) {
     const int64_t ia = __ldg(&a.rb[r]), ib = __ldg(&a.rb[r + 1]);
     int64_t i = ia;
     while (i < ib) {
-      const int v = __ldg(&a.ihead[i]);
+      // a run of in-edges whose heads have short out-lists goes together
+      int v = 0, db = 0, dd = 0;
+      if (i + lane < ib) {
+        v = __ldg(&a.ihead[i + lane]);
+        const int64_t o0 = __ldg(&a.offp[v]);
+        db = (int)o0;
+        dd = (int)(__ldg(&a.offp[v + 1]) - o0);
+      }
+      const unsigned other = __ballot_sync(TR_FULL, i + lane >= ib || dd >= a.stage_min);
+      const int run = other ? __ffs(other) - 1 : 32;
+      if (run > 0) {
+        mixed_walk(a, i, run, db, dd);
+        i += run;
+        continue;
+      }
+      v = __shfl_sync(TR_FULL, v, 0);
       const int64_t vbeg = __ldg(&a.inoff[v]), vend = __ldg(&a.inoff[v + 1]);
       const int64_t iend = min(ib, vend);
       const int64_t bv = __ldg(&a.offp[v]);
       const int dv = (int)(__ldg(&a.offp[v + 1]) - bv);
       const int64_t i0 = i;
       i = iend;
-      if (dv == 0) continue;  // no w above v: no triangle has v in the middle
       const bool whole = i0 == vbeg && iend == vend;
-      if (dv < a.stage_min) {
-        // a few entries: search the (L1-cached) global list; staging costs
-        // more than the probes of so short a head save
-        head_walk<kSearch>(a, i0, iend, bv, dv, __ldg(&a.adjp[bv + dv - 1]), nullptr, nullptr,
-                           nullptr, 0, 0);
-      } else if (dv <= a.stage_max) {
+      if (dv <= a.stage_max) {
         int lg = 32 - __clz(max(8 * dv - 1, 63));  // ceil(log2(8 dv)), at least 6
         lg = min(lg, 11);
         const int S = 1 << lg, sh = 32 - lg;
@@ -601,10 +709,8 @@ __global__ void k_walk_cost(int64_t m, const int64_t *offp, const int32_t *adjp,
 // of a few heavy edges still keeps every warp of the block busy.
 constexpr int kListU = 4;
 constexpr int kLBlock = 512;
-constexpr int kLCap = 16384;       // shared cursor counters per range (64 KB)
-constexpr int kLEdgeCost = 4;      // range cost per edge (next to its records)
-constexpr int64_t kLRangeCost = (int64_t)kLCap * kLEdgeCost / 2;
-constexpr int64_t kLMinCost = 512;
+constexpr int kLCap = kListCounters;
+constexpr int kLEdgeCost = kListEdgeCost;
 
 struct ListPass {
   int64_t m, n;
@@ -845,48 +951,78 @@ int launch_list_walk(Arena &A, ListArgs a, const SupportCfg &cfg, cudaStream_t s
   return TRUSS_OK;
 }
 
-int launch_walk_v(Arena &A, SupVArgs a, const SupportCfg &cfg, cudaStream_t s) {
+constexpr size_t kWalkSmem = (size_t)(kBlock / 32) * kHeadSmem;
+
+// Resident blocks of the walk over the whole device.
+int walk_grid(const SupportCfg &cfg, int *grid) {
   int dev = 0, sms = cfg.sms;
   TR_CUDA(cudaGetDevice(&dev));
   if (sms <= 0) TR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const size_t smem = (size_t)(kBlock / 32) * kHeadSmem;
   TR_CUDA(cudaFuncSetAttribute(k_support_v, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
+                               (int)kWalkSmem));
   int occ = 0;
-  TR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_support_v, kBlock, smem));
+  TR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_support_v, kBlock, kWalkSmem));
   if (occ < 1) occ = 1;
-  const int grid = sms * occ;
-  const int64_t warps = (int64_t)grid * (kBlock / 32);
-  int64_t P = a.W / (cfg.range_work > 0 ? cfg.range_work : kRangeWork);
-  if (P < warps) P = warps;
-  if (P > a.m) P = a.m > 0 ? a.m : 1;
-  a.P = P;
-  int64_t *rb = A.get<int64_t>(P + 1);
-  if (!rb) return TRUSS_ENOMEM;
-  k_range_bounds<<<grid_for(P + 1, 256, 152 * 8), 256, 0, s>>>(a.m, P, a.W, a.wpre, rb);
-  TR_LAUNCHED();
-  a.rb = rb;
+  *grid = sms * occ;
+  return TRUSS_OK;
+}
+
+// The walk; its ranges are cut here unless a.rb has them.
+int launch_walk_v(Arena &A, SupVArgs a, const SupportCfg &cfg, cudaStream_t s) {
+  int grid = 0;
+  TR_TRY(walk_grid(cfg, &grid));
+  if (!a.rb) {
+    const int64_t warps = (int64_t)grid * (kBlock / 32);
+    int64_t P = a.W / walk_range_work(cfg);
+    if (P < warps) P = warps;
+    if (P > a.m) P = a.m > 0 ? a.m : 1;
+    a.P = P;
+    int64_t *rb = A.get<int64_t>(P + 1);
+    if (!rb) return TRUSS_ENOMEM;
+    k_range_bounds<<<grid_for(P + 1, 256, 152 * 8), 256, 0, s>>>(a.m, P, a.W, a.wpre, rb);
+    TR_LAUNCHED();
+    a.rb = rb;
+  }
   a.stage_max = cfg.stage_max > 0 && cfg.stage_max < kHeadCap ? cfg.stage_max : kHeadCap;
   a.hash_max = kHashOnlyCap;
   a.stage_min = kStageMin;
-  k_support_v<<<grid, kBlock, smem, s>>>(a);
+  k_support_v<<<grid, kBlock, kWalkSmem, s>>>(a);
   TR_LAUNCHED();
   return TRUSS_OK;
 }
 
 }  // namespace
 
-int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, cudaStream_t s) {
+int walk_edge_cost(const SupportCfg &cfg) {
+  return cfg.pair_cost > 0 ? cfg.pair_cost : cfg.pair_cost < 0 ? 0 : kEdgeCost;
+}
+
+int64_t walk_range_work(const SupportCfg &cfg) {
+  return cfg.range_work > 0 ? cfg.range_work : kRangeWork;
+}
+
+int walk_warps(const SupportCfg &cfg, int64_t *warps) {
+  int grid = 0;
+  TR_TRY(walk_grid(cfg, &grid));
+  *warps = (int64_t)grid * (kBlock / 32);
+  return TRUSS_OK;
+}
+
+namespace {
+
+// Edges grouped by head, walk costs and record bounds with their prefixes, by
+// device-wide sorts and scans.
+int prepare_walk(Arena &A, const Csr &g, const SupportCfg &cfg, SupportPrep *out,
+                 cudaStream_t s) {
   const int64_t m = g.m, n = g.n;
-  int32_t *supA = A.get<int32_t>(m), *supB = A.get<int32_t>(m), *sup = A.get<int32_t>(m);
-  int64_t *sup64 = A.get<int64_t>(m + 1), *toff = A.get<int64_t>(m + 1);
+  int32_t *supA = A.get<int32_t>(m), *supB = A.get<int32_t>(m);
   int64_t *wcost = A.get<int64_t>(m + 1), *wpre = A.get<int64_t>(m + 1);
   int64_t *wbound = A.get<int64_t>(m + 1), *tbpre = A.get<int64_t>(m + 1);
   int64_t *hcnt = A.get<int64_t>(n + 1);
   int64_t *inoff = A.get<int64_t>(n + 1);
   int32_t *inedge = A.get<int32_t>(m), *ihead = A.get<int32_t>(m);
-  if (!supA || !supB || !sup || !sup64 || !toff || !wcost || !wpre || !wbound || !tbpre ||
-      !hcnt || !inoff || !inedge || !ihead)
+  if (!supA || !supB || !wcost || !wpre || !wbound || !tbpre || !hcnt || !inoff || !inedge ||
+      !ihead)
     return TRUSS_ENOMEM;
   TR_CUDA(cudaMemsetAsync(supA, 0, sizeof(int32_t) * m, s));
   TR_CUDA(cudaMemsetAsync(supB, 0, sizeof(int32_t) * m, s));
@@ -913,7 +1049,7 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, 
     TR_TRY(exclusive_sum_i64(tmp, &tb, hcnt, inoff, n + 1, s));
     TR_TRY(sort_pairs_u32(tmp, &tb3, (const uint32_t *)g.adjp, (uint32_t *)ihead, ids, inedge, m,
                           0, hbits, s));
-    const int ec = cfg.pair_cost > 0 ? cfg.pair_cost : cfg.pair_cost < 0 ? 0 : kEdgeCost;
+    const int ec = walk_edge_cost(cfg);
     k_walk_cost_v<<<grid_for(m + 1, 256, 152 * 16), 256, 0, s>>>(m, g.offp, g.adjp, g.esrc,
                                                                   inedge, wcost, wbound, ec);
     TR_LAUNCHED();
@@ -924,6 +1060,30 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, 
       TR_CUDA(cudaMemcpyAsync(&R, tbpre + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     TR_CUDA(cudaStreamSynchronize(s));
   }
+  out->supA = supA;
+  out->supB = supB;
+  out->inedge = inedge;
+  out->ihead = ihead;
+  out->inoff = inoff;
+  out->wcost = wcost;
+  out->wpre = wpre;
+  out->tbpre = tbpre;
+  out->W = W;
+  out->R = R;
+  return TRUSS_OK;
+}
+
+}  // namespace
+
+int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportPrep &ready,
+                SupportOut *out, cudaStream_t s) {
+  const int64_t m = g.m, n = g.n;
+  int32_t *sup = A.get<int32_t>(m);
+  int64_t *toff = A.get<int64_t>(m + 1);
+  if (!sup || !toff) return TRUSS_ENOMEM;
+  SupportPrep pre = ready;
+  if (!pre.valid) TR_TRY(prepare_walk(A, g, cfg, &pre, s));
+  const int64_t W = pre.W, R = pre.R;
   // Records need 8 R bytes now, and the lists later 24 bytes per triangle
   // when they are whole, 16 with the own parts left in the records, plus a
   // few words per edge for the list passes and the peel.  The walk records
@@ -935,22 +1095,16 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, 
   int32_t *cuv = nullptr;
   bool in_place = false;
   if (cfg.records && R > 0) {
-    size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-      cudaGetLastError();
-      fr = 0;
-    }
-    const double avail = (double)A.headroom(fr);
     const double need_whole = 1.05 * (32.0 * (double)R + 20.0 * (double)m);
     const double need_in_place = 1.05 * (24.0 * (double)R + 36.0 * (double)m);
-    const bool use = cfg.full_lists ? need_whole < avail : need_in_place < avail;
+    const bool use = A.has_room(cfg.full_lists ? need_whole : need_in_place);
     if (use) {
       recs = A.get<int2>(R);
-      cuv = A.get<int32_t>(m);
+      cuv = pre.cuv ? pre.cuv : A.get<int32_t>(m);
       if (!recs || !cuv) {
         recs = nullptr;
         cuv = nullptr;
-      } else {
+      } else if (!pre.cuv) {
         TR_CUDA(cudaMemsetAsync(cuv, 0, sizeof(int32_t) * m, s));
       }
     }
@@ -962,53 +1116,57 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, SupportOut *out, 
     a.offp = g.offp;
     a.adjp = g.adjp;
     a.esrc = g.esrc;
-    a.inedge = inedge;
-    a.ihead = ihead;
-    a.inoff = inoff;
-    a.wcost = wcost;
-    a.wpre = wpre;
+    a.inedge = pre.inedge;
+    a.ihead = pre.ihead;
+    a.inoff = pre.inoff;
+    a.wcost = pre.wcost;
+    a.wpre = pre.wpre;
+    a.rb = pre.rb;
     a.W = W;
-    a.ecost = cfg.pair_cost > 0 ? cfg.pair_cost : cfg.pair_cost < 0 ? 0 : kEdgeCost;
-    a.supA = supA;
-    a.supB = supB;
-    a.tbpre = tbpre;
+    a.P = pre.P;
+    a.ecost = walk_edge_cost(cfg);
+    a.supA = pre.supA;
+    a.supB = pre.supB;
+    a.tbpre = pre.tbpre;
     a.tb = recs;
     a.cuv = cuv;
     TR_TRY(launch_walk_v(A, a, cfg, s));
   }
-  k_sum<<<grid_for(m + 1, 256, 152 * 16), 256, 0, s>>>(m, supA, supB, sup, sup64);
-  TR_LAUNCHED();
-  size_t tb = 0;
-  TR_TRY(exclusive_sum_i64(nullptr, &tb, sup64, toff, m + 1, s));
-  void *tmp = A.alloc(tb);
-  if (!tmp) return TRUSS_ENOMEM;
-  TR_TRY(exclusive_sum_i64(tmp, &tb, sup64, toff, m + 1, s));
   int64_t total = 0;
-  TR_CUDA(cudaMemcpyAsync(&total, toff + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  TR_CUDA(cudaStreamSynchronize(s));
+  if (pre.valid) {
+    TR_TRY(small_offsets(A, g, pre, recs ? cuv : nullptr, cfg.sms, sup, toff, &total, &out->small,
+                         s));
+  } else {
+    int64_t *sup64 = A.get<int64_t>(m + 1);
+    if (!sup64) return TRUSS_ENOMEM;
+    k_sum<<<grid_for(m + 1, 256, 152 * 16), 256, 0, s>>>(m, pre.supA, pre.supB, sup, sup64);
+    TR_LAUNCHED();
+    size_t tb = 0;
+    TR_TRY(exclusive_sum_i64(nullptr, &tb, sup64, toff, m + 1, s));
+    void *tmp = A.alloc(tb);
+    if (!tmp) return TRUSS_ENOMEM;
+    TR_TRY(exclusive_sum_i64(tmp, &tb, sup64, toff, m + 1, s));
+    TR_CUDA(cudaMemcpyAsync(&total, toff + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    TR_CUDA(cudaStreamSynchronize(s));
+  }
   out->sup = sup;
-  out->supA = supA;
+  out->supA = pre.supA;
   out->toff = toff;
   out->walk = W;
   out->entries = total;
-  out->inedge = inedge;
-  out->inoff = inoff;
+  out->inedge = pre.inedge;
+  out->inoff = pre.inoff;
   if (recs && !cfg.full_lists) {
     if (cfg.in_place) {
       in_place = true;
     } else {
       // whole lists: 3T entries, the peel's work items (up to 3T/16 + m, two
       // queues) and about 100 B per edge for the list passes and the peel
-      size_t fr = 0, tot = 0;
-      if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-        cudaGetLastError();
-        fr = 0;
-      }
       const double tri = (double)(total / 3);
-      in_place = !(1.05 * (30.0 * tri + 100.0 * (double)m) < (double)A.headroom(fr));
+      in_place = !A.has_room(1.05 * (30.0 * tri + 100.0 * (double)m));
     }
   }
-  out->tbpre = recs ? tbpre : nullptr;
+  out->tbpre = recs ? pre.tbpre : nullptr;
   out->records = recs ? R : 0;
   out->tb = recs;
   out->cuv = recs ? cuv : nullptr;
@@ -1026,10 +1184,11 @@ int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &s
   if (so.tb) {
     const bool in_place = so.in_place;
     if (tids && in_place) return TRUSS_EINVAL;  // triangle ids come with whole lists
-    unsigned long long *cur = A.get<unsigned long long>(m);
-    int *err = A.get<int>(1);
-    if (!cur || !err) return TRUSS_ENOMEM;
-    TR_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+    const bool ready = so.small.cur != nullptr && !in_place;  // small graph: all prepared
+    int *err = &g.zero->list_err;
+    unsigned long long *next = g.zero->list_next;
+    unsigned long long *cur = ready ? so.small.cur : A.get<unsigned long long>(m);
+    if (!cur) return TRUSS_ENOMEM;
     const int64_t rest = list_rest_entries(so);
     if (in_place) {
       int64_t *len = A.get<int64_t>(m + 1), *roff = A.get<int64_t>(m + 1);
@@ -1047,41 +1206,37 @@ int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &s
       out->own_off = so.tbpre;
       out->own_cnt = so.cuv;
       out->off = roff;
-    } else {
+    } else if (!ready) {
       k_cursors_rec<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, so.toff, so.cuv, cur);
       TR_LAUNCHED();
     }
-    // vertex ranges of about kLRangeCost: pass 1 over owners (edge order),
-    // pass 2 over heads (the support walk's in-edge index)
-    const int64_t n = g.n, tri = so.entries / 3;
-    int64_t *c1 = A.get<int64_t>(m + 1), *c2 = A.get<int64_t>(m + 1);
-    int64_t *p1 = A.get<int64_t>(m + 1), *p2 = A.get<int64_t>(m + 1);
-    // Ranges of kLRangeCost leave most blocks idle below some 10 M triangles:
-    // smaller graphs take four ranges per block, but none under kLMinCost
-    // (list passes of the 4,096-vertex graph 62 us, now LP_TINY us; of R-MAT
-    // scale 15 163 us, now LP_SMALL us).
-    const int64_t total = tri + 2 * kLEdgeCost * m, fit = total / (4 * 2 * 152);
-    const int64_t rc = fit > kLRangeCost ? kLRangeCost : fit < kLMinCost ? kLMinCost : fit;
-    const int64_t nr1 = (tri + kLEdgeCost * m) / rc + 1;
-    const int64_t nr2 = total / rc + 1;
-    int64_t *vb1 = A.get<int64_t>(nr1 + 1), *vb2 = A.get<int64_t>(nr2 + 1);
-    unsigned long long *next = A.get<unsigned long long>(2);
-    if (!c1 || !c2 || !p1 || !p2 || !vb1 || !vb2 || !next) return TRUSS_ENOMEM;
-    k_list_costs<<<grid_for(m + 1, 256, 152 * 16), 256, 0, s>>>(m, so.cuv, so.inedge, c1, c2);
-    TR_LAUNCHED();
-    size_t tb = 0;
-    TR_TRY(exclusive_sum_i64(nullptr, &tb, c1, p1, m + 1, s));
-    void *tmp = A.alloc(tb);
-    if (!tmp) return TRUSS_ENOMEM;
-    TR_TRY(exclusive_sum_i64(tmp, &tb, c1, p1, m + 1, s));
-    TR_TRY(exclusive_sum_i64(tmp, &tb, c2, p2, m + 1, s));
-    k_list_ranges<<<grid_for(nr1 + 1, 256, 152 * 8), 256, 0, s>>>(n, nr1, p1, g.offp, g.offp,
-                                                                    false, rc, vb1);
-    TR_LAUNCHED();
-    k_list_ranges<<<grid_for(nr2 + 1, 256, 152 * 8), 256, 0, s>>>(n, nr2, p2, so.inoff, g.offp,
-                                                                    true, rc, vb2);
-    TR_LAUNCHED();
-    TR_CUDA(cudaMemsetAsync(next, 0, 2 * sizeof(unsigned long long), s));
+    // vertex ranges: pass 1 over owners (edge order), pass 2 over heads (the
+    // support walk's in-edge index)
+    const int64_t n = g.n;
+    const ListRanges lr = list_ranges(so.entries / 3, m);
+    int64_t *p1 = so.small.p1, *p2 = so.small.p2, *vb1 = so.small.vb1, *vb2 = so.small.vb2;
+    if (!ready) {
+      int64_t *c1 = A.get<int64_t>(m + 1), *c2 = A.get<int64_t>(m + 1);
+      p1 = A.get<int64_t>(m + 1);
+      p2 = A.get<int64_t>(m + 1);
+      vb1 = A.get<int64_t>(lr.n1 + 1);
+      vb2 = A.get<int64_t>(lr.n2 + 1);
+      if (!c1 || !c2 || !p1 || !p2 || !vb1 || !vb2) return TRUSS_ENOMEM;
+      k_list_costs<<<grid_for(m + 1, 256, 152 * 16), 256, 0, s>>>(m, so.cuv, so.inedge, c1, c2);
+      TR_LAUNCHED();
+      size_t tb = 0;
+      TR_TRY(exclusive_sum_i64(nullptr, &tb, c1, p1, m + 1, s));
+      void *tmp = A.alloc(tb);
+      if (!tmp) return TRUSS_ENOMEM;
+      TR_TRY(exclusive_sum_i64(tmp, &tb, c1, p1, m + 1, s));
+      TR_TRY(exclusive_sum_i64(tmp, &tb, c2, p2, m + 1, s));
+      k_list_ranges<<<grid_for(lr.n1 + 1, 256, 152 * 8), 256, 0, s>>>(n, lr.n1, p1, g.offp, g.offp,
+                                                                      false, lr.cost, vb1);
+      TR_LAUNCHED();
+      k_list_ranges<<<grid_for(lr.n2 + 1, 256, 152 * 8), 256, 0, s>>>(
+          n, lr.n2, p2, so.inoff, g.offp, true, lr.cost, vb2);
+      TR_LAUNCHED();
+    }
     int dev = 0, sms = cfg.sms;
     TR_CUDA(cudaGetDevice(&dev));
     if (sms <= 0) TR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1111,29 +1266,24 @@ int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &s
     lp.err = err;
     lp.vb = vb1;
     lp.pre = p1;
-    lp.nranges = nr1;
+    lp.nranges = lr.n1;
     lp.next = next;
     k_lists_pass<false><<<sms * occ, kLBlock, smem, s>>>(lp);
     TR_LAUNCHED();
     lp.vb = vb2;
     lp.pre = p2;
-    lp.nranges = nr2;
+    lp.nranges = lr.n2;
     lp.next = next + 1;
     k_lists_pass<true><<<sms * occ, kLBlock, smem, s>>>(lp);
     TR_LAUNCHED();
-    int h_err = 0;
-    TR_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    TR_CUDA(cudaStreamSynchronize(s));
-    return h_err != 0 ? TRUSS_ECHECK : TRUSS_OK;
+    return TRUSS_OK;
   }
   // No records (short of memory): walk the graph again, owner by owner, and
   // write the lists directly.  Its ranges need the owner-centric walk cost.
   unsigned long long *curA = A.get<unsigned long long>(m), *curB = A.get<unsigned long long>(m);
   int64_t *wcost = A.get<int64_t>(m + 1), *wpre = A.get<int64_t>(m + 1);
   int64_t *wbound = A.get<int64_t>(m + 1);
-  int *err = A.get<int>(1);
-  if (!curA || !curB || !wcost || !wpre || !wbound || !err) return TRUSS_ENOMEM;
-  TR_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+  if (!curA || !curB || !wcost || !wpre || !wbound) return TRUSS_ENOMEM;
   const int ec = cfg.pair_cost > 0 ? cfg.pair_cost : cfg.pair_cost < 0 ? 0 : kEdgeCost;
   k_walk_cost<<<grid_for(m + 1, 256, 152 * 16), 256, 0, s>>>(m, g.offp, g.adjp, g.esrc, wcost,
                                                               wbound, ec);
@@ -1160,12 +1310,8 @@ int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &s
   a.curB = curB;
   a.pairs = pairs;
   a.entries = so.entries;
-  a.err = err;
-  TR_TRY(launch_list_walk(A, a, cfg, s));
-  int h_err = 0;
-  TR_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
-  TR_CUDA(cudaStreamSynchronize(s));
-  return h_err != 0 ? TRUSS_ECHECK : TRUSS_OK;
+  a.err = &g.zero->list_err;
+  return launch_list_walk(A, a, cfg, s);
 }
 
 }  // namespace tr

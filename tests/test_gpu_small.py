@@ -1,0 +1,117 @@
+"""The launches that build small graphs in one kernel, and the support walk's
+mixed runs of short out-lists, at the sizes where they can go wrong: edges of
+tiles and warps, degrees around the counted ones, the largest size taken and
+one more.  Against the CPU oracle, or against the general path (which a context
+with a wait limit takes); all outputs are integers and compared exactly."""
+import numpy as np
+import pytest
+
+import graphgen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SMALL_ROWS = 5 << 19  # csrc/small.cu: kSmallRows
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1205_6693_gb300 import truss as T
+    c = T.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.fixture(scope="module")
+def general():
+    from paper_1205_6693_gb300 import truss as T
+    c = T.Context(0, wait_limit_ns=4_000_000_000)
+    yield c
+    c.close()
+
+
+def run(ctx, n, s, d):
+    sup, tr = torch.full_like(s, -7), torch.full_like(s, -7)
+    k = ctx.decompose(n, s, d, sup, tr)
+    only = torch.full_like(s, -7)
+    ctx.support(n, s, d, only)
+    assert torch.equal(only, sup)
+    return sup.cpu().numpy(), tr.cpu().numpy(), k
+
+
+def check(ctx, n, src, dst):
+    s = torch.from_numpy(np.ascontiguousarray(src, np.int32)).cuda()
+    d = torch.from_numpy(np.ascontiguousarray(dst, np.int32)).cuda()
+    ref = oracle.truss(n, src, dst)
+    sup, tr, k = run(ctx, n, s, d)
+    assert np.array_equal(sup, ref.support) and np.array_equal(tr, ref.truss) and k == ref.kmax
+
+
+@pytest.mark.parametrize("rows", [1, 2, 31, 33, 511, 512, 513, 1023, 1025, 8191, 60_001])
+def test_row_counts_around_tiles(ctx, rows):
+    # random pairs of a dense and a sparse graph, self-loops and reversed
+    # duplicates among them
+    for n in (max(2, rows // 6), rows + 3):
+        rng = np.random.default_rng(rows)
+        check(ctx, n, rng.integers(0, n, rows), rng.integers(0, n, rows))
+
+
+@pytest.mark.parametrize("hub", [254, 255, 256, 257, 600])
+def test_degrees_around_the_counted_ones(ctx, hub):
+    # hubs of equal degree, joined in a clique, with leaves of their own
+    h = 6
+    a, b = np.triu_indices(h, 1)
+    leaves = hub - (h - 1)
+    src = np.concatenate([a, np.repeat(np.arange(h), leaves)])
+    dst = np.concatenate([b, h + np.arange(h * leaves)])
+    perm = graphgen.permutation(h + h * leaves, seed=hub, stream=1)
+    check(ctx, h + h * leaves, perm[src], perm[dst])
+
+
+@pytest.mark.parametrize("sizes", [[31, 32, 33], [34, 64, 66], [3, 4, 5, 150, 170]])
+def test_out_lists_around_the_mixed_limit(ctx, sizes):
+    # a clique K_s has out-lists of every length below s: runs of heads on
+    # both sides of the staging limit, and walks longer than 128 entries
+    n = 4000
+    src, dst = graphgen.er(n, 9000, seed=sizes[0])
+    perm = graphgen.permutation(n, seed=sizes[0], stream=1)
+    check(ctx, n, *graphgen.add_cliques(src, dst, perm[: sum(sizes)], sizes))
+
+
+@pytest.mark.parametrize("rows", [SMALL_ROWS, SMALL_ROWS + 1])
+@pytest.mark.parametrize("kind", ["rmat", "random"])
+def test_largest_size_and_one_more(ctx, general, rows, kind):
+    if kind == "rmat":
+        n, (s, d) = 1 << 18, graphgen.rmat_raw_cuda(18, rows, seed=5)
+    else:
+        n, g = SMALL_ROWS, torch.Generator(device="cuda").manual_seed(5)
+        s = torch.randint(0, n, (rows,), dtype=torch.int32, generator=g, device="cuda")
+        d = torch.randint(0, n, (rows,), dtype=torch.int32, generator=g, device="cuda")
+    a, b = run(ctx, n, s, d), run(general, n, s, d)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1]) and a[2] == b[2]
+    assert ctx.stats()["triangles"] == general.stats()["triangles"]
+
+
+def test_small_batch_and_bad_ids(ctx):
+    from paper_1205_6693_gb300 import truss as T
+    G = 30
+    ns, off, src, dst = graphgen.batch(G)
+    assert off[-1] <= SMALL_ROWS
+    s, d = torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()
+    sup, tr = torch.empty_like(s), torch.empty_like(s)
+    kmax = torch.empty(G, dtype=torch.int32, device="cuda")
+    ctx.decompose_batch(ns, off, s, d, sup, tr, kmax)
+    sup, tr, kmax = sup.cpu().numpy(), tr.cpu().numpy(), kmax.cpu().numpy()
+    for g in range(G):
+        a, b = off[g], off[g + 1]
+        ref = oracle.truss(int(ns[g]), src[a:b], dst[a:b])
+        assert np.array_equal(sup[a:b], ref.support) and np.array_equal(tr[a:b], ref.truss)
+        assert kmax[g] == ref.kmax
+    # an id beyond its own graph is refused though it lies in the union
+    bad = src.copy()
+    bad[off[3]] = ns[3]
+    sb = torch.from_numpy(bad).cuda()
+    with pytest.raises(T.TrussError) as ei:
+        ctx.decompose_batch(ns, off, sb, d, torch.empty_like(s), torch.empty_like(s))
+    assert ei.value.code == T.TRUSS_EINVAL
