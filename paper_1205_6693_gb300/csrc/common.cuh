@@ -82,6 +82,40 @@ __device__ __forceinline__ int warp_owner(int P, int t) {
   return o;
 }
 
+// Position of the r-th set bit of m (r from 0, below the number of set bits).
+__device__ __forceinline__ int nth_set_bit(unsigned m, int r) {
+  int pos = 0;
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) {
+    const int low = __popc(m & ((1u << s) - 1u));
+    if (r >= low) {
+      r -= low;
+      pos += s;
+      m >>= s;
+    }
+  }
+  return pos;
+}
+
+// Work of different lengths spread over a warp: lane l < n (n non-empty
+// pieces) holds piece l, which takes the steps [S, S + len) of all pieces laid
+// end to end.  owner() finds the piece of each lane's step of the window
+// [tr, tr + 32), for consecutive windows from 0 on: the pieces that start in
+// the window set one bit each, so it takes one warp reduction and a bit count
+// where a search through the prefix takes five dependent shuffles.
+struct FlatWork {
+  int S, len;
+  int before = 0;  // pieces that started before the window
+  __device__ __forceinline__ int owner(int tr) {
+    const int rel = S - tr;
+    const unsigned bit = len > 0 && (unsigned)rel < 32u ? 1u << rel : 0u;
+    const unsigned mask = __reduce_or_sync(TR_FULL, bit);
+    const int o = before + __popc(mask & (0xFFFFFFFFu >> (31 - lane_id()))) - 1;
+    before += __popc(mask);
+    return o;
+  }
+};
+
 // Warp-aggregated append: every lane with `pred` gets a distinct slot in a
 // buffer whose fill counter is *cnt; returns the slot (or -1).  All lanes of
 // the warp must call it.

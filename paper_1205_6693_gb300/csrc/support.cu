@@ -261,7 +261,11 @@ __device__ __forceinline__ int find_in_out(int w, const int32_t *Ls, const unsig
 
 // Walks of at most kShortWalk entries are spread over the lanes, several
 // edges per warp step; longer ones take the warp one edge at a time.
-constexpr int kShortWalk = 128;
+// Support stage at 32 / 64 / 128 / 256: R-MAT scale 20 8.17 / 8.25 / 8.61 /
+// 9.53 ms, 40 M-edge Chung-Lu 11.3 / 11.1 / 11.2 / 11.9, 10 M rows 1.88 / 1.85 /
+// 1.98 / 2.05.  (With each step's owner searched by five shuffles, at 128: 9.40,
+// 11.95 and 2.21 ms.)
+constexpr int kShortWalk = 64;
 constexpr int kFlatU = 4;  // flattened steps whose loads are issued together
 
 // One hit of the walk: triangle (u, v, w) with e_uw = euw and e_vw at
@@ -273,6 +277,13 @@ __device__ __forceinline__ void count_hit(const SupVArgs &a, int32_t *Cs, int64_
   else atomicAdd(&a.supB[bv + q], 1);
   atomicAdd(&a.supA[euw], 1);
   if (a.tb) a.tb[slot] = make_int2((int)euw, (int)(bv + q));
+}
+
+// Bits [lo, hi) of hm (bounds outside 0 .. 32 cut).
+__device__ __forceinline__ int own_hits(unsigned hm, int lo, int hi) {
+  if (hi <= 0 || lo >= 32 || hi <= lo) return 0;
+  const unsigned below = hi >= 32 ? 0xFFFFFFFFu : (1u << hi) - 1u;
+  return __popc(hm & below & (lo > 0 ? ~((1u << lo) - 1u) : 0xFFFFFFFFu));
 }
 
 // The in-edges inedge[i0 .. i1) of head v (bv = offp[v], dv = |out(v)|).
@@ -291,24 +302,28 @@ __device__ __forceinline__ void head_walk(const SupVArgs &a, int64_t i0, int64_t
     const int len = valid ? (int)(__ldg(&a.wcost[j]) - a.ecost) : 0;  // out(u) after v
     const int64_t rb = (valid && a.tb) ? __ldg(&a.tbpre[e]) : 0;
 
-    // short walks, flattened: step t of the warp is entry t - base(o) of
-    // the walk of lane o = the owner of t (base = exclusive prefix of sl)
+    // short walks, flattened: the non-empty ones move to the first lanes, and
+    // a lane's step of the warp is an entry of its owner's walk
     const bool shrt = len <= kShortWalk;
-    const int sl = shrt ? len : 0;
+    const unsigned ne = __ballot_sync(TR_FULL, shrt && len > 0);
+    const int nw = __popc(ne), src = nth_set_bit(ne, lane < nw ? lane : 0);
+    const int fe = __shfl_sync(TR_FULL, e, src);
+    const int64_t frb = __shfl_sync(TR_FULL, rb, src);
+    int sl = __shfl_sync(TR_FULL, len, src);
+    sl = lane < nw ? sl : 0;
     const int P = warp_incl_scan(sl);
-    const int total = __shfl_sync(TR_FULL, P, 31);
+    const int total = nw > 0 ? __shfl_sync(TR_FULL, P, 31) : 0;
+    FlatWork fw{P - sl, sl};
     int mycnt = 0;  // triangles found so far for this lane's (short) edge
     for (int t0 = 0; t0 < total; t0 += 32 * kFlatU) {
-      int w[kFlatU], own[kFlatU], bo[kFlatU];
+      int w[kFlatU], own[kFlatU], bo[kFlatU], eo[kFlatU];
 #pragma unroll
       for (int k = 0; k < kFlatU; k++) {
         const int t = t0 + k * 32 + lane;
-        const bool act = t < total;
-        own[k] = warp_owner(P, act ? t : total - 1);
-        const int Po = __shfl_sync(TR_FULL, P, own[k]), so = __shfl_sync(TR_FULL, sl, own[k]);
-        const int eo = __shfl_sync(TR_FULL, e, own[k]);
-        bo[k] = Po - so;
-        w[k] = act ? __ldg(&a.adjp[(int64_t)eo + 1 + (t - bo[k])]) : INT_MAX;
+        own[k] = fw.owner(t0 + k * 32);
+        bo[k] = __shfl_sync(TR_FULL, fw.S, own[k]);
+        eo[k] = __shfl_sync(TR_FULL, fe, own[k]);
+        w[k] = t < total ? __ldg(&a.adjp[(int64_t)eo[k] + 1 + (t - bo[k])]) : INT_MAX;
       }
 #pragma unroll
       for (int k = 0; k < kFlatU; k++) {
@@ -318,30 +333,20 @@ __device__ __forceinline__ void head_walk(const SupVArgs &a, int64_t i0, int64_t
         const unsigned hm = __ballot_sync(TR_FULL, q >= 0);
         if (hm == 0) continue;
         const int prior = __shfl_sync(TR_FULL, mycnt, own[k]);
-        const int64_t tbase = __shfl_sync(TR_FULL, rb, own[k]);
-        const int eo = __shfl_sync(TR_FULL, e, own[k]);
+        const int64_t tbase = __shfl_sync(TR_FULL, frb, own[k]);
         if (q >= 0) {
           // lanes of this round that walk the same edge: steps [bo, bo + so)
           const int lo = max(bo[k] - tr, 0);
           const unsigned below = hm & lt & ~((1u << lo) - 1u);
-          const int64_t euw = (int64_t)eo + 1 + (tr + lane - bo[k]);
+          const int64_t euw = (int64_t)eo[k] + 1 + (tr + lane - bo[k]);
           count_hit<MODE>(a, Cs, bv, q, euw, tbase + prior + __popc(below));
         }
-        // owners add this round's hits of their own walk
-        if (sl > 0) {
-          const int lo = P - sl - tr, hi = P - 1 - tr;
-          if (hi >= 0 && lo <= 31) {
-            const int l0 = max(lo, 0), l1 = min(hi, 31);
-            const unsigned seg = (l1 == 31 ? 0xFFFFFFFFu : ((1u << (l1 + 1)) - 1u)) &
-                                 ~((1u << l0) - 1u);
-            mycnt += __popc(hm & seg);
-          }
-        }
+        mycnt += own_hits(hm, fw.S - tr, P - tr);
       }
     }
-    if (valid && shrt) {
-      if (a.tb) a.cuv[e] = mycnt;
-      if (mycnt) atomicAdd(&a.supA[e], mycnt);
+    if (mycnt) {  // cuv starts at zero
+      if (a.tb) a.cuv[fe] = mycnt;
+      atomicAdd(&a.supA[fe], mycnt);
     }
 
     // long walks: the whole warp on one edge, stopping past max out(v)
@@ -405,53 +410,50 @@ __device__ __forceinline__ void mixed_walk(const SupVArgs &a, int64_t i0, int cn
     return q < d && __ldg(&a.adjp[b + q]) == w ? q : -1;
   };
   const bool shrt = len <= kShortWalk;
-  const int sl = shrt ? len : 0;
+  const unsigned ne = __ballot_sync(TR_FULL, shrt && len > 0);
+  const int nw = __popc(ne), src = nth_set_bit(ne, lane < nw ? lane : 0);
+  const int fe = __shfl_sync(TR_FULL, e, src), fb = __shfl_sync(TR_FULL, bv, src);
+  const int fd = __shfl_sync(TR_FULL, dv, src), fm = __shfl_sync(TR_FULL, vmax, src);
+  const int64_t frb = __shfl_sync(TR_FULL, rb, src);
+  int sl = __shfl_sync(TR_FULL, len, src);
+  sl = lane < nw ? sl : 0;
   const int P = warp_incl_scan(sl);
-  const int total = __shfl_sync(TR_FULL, P, 31);
+  const int total = nw > 0 ? __shfl_sync(TR_FULL, P, 31) : 0;
+  FlatWork fw{P - sl, sl};
   int mycnt = 0;  // triangles found so far for this lane's (short) edge
   for (int t0 = 0; t0 < total; t0 += 32 * kFlatU) {
-    int w[kFlatU], own[kFlatU], bo[kFlatU];
+    int w[kFlatU], own[kFlatU], bo[kFlatU], eo[kFlatU];
 #pragma unroll
     for (int k = 0; k < kFlatU; k++) {
       const int t = t0 + k * 32 + lane;
-      const bool act = t < total;
-      own[k] = warp_owner(P, act ? t : total - 1);
-      bo[k] = __shfl_sync(TR_FULL, P - sl, own[k]);
-      const int eo = __shfl_sync(TR_FULL, e, own[k]);
-      w[k] = act ? __ldg(&a.adjp[(int64_t)eo + 1 + (t - bo[k])]) : INT_MAX;
+      own[k] = fw.owner(t0 + k * 32);
+      bo[k] = __shfl_sync(TR_FULL, fw.S, own[k]);
+      eo[k] = __shfl_sync(TR_FULL, fe, own[k]);
+      w[k] = t < total ? __ldg(&a.adjp[(int64_t)eo[k] + 1 + (t - bo[k])]) : INT_MAX;
     }
 #pragma unroll
     for (int k = 0; k < kFlatU; k++) {
       const int tr = t0 + k * 32;  // step of lane 0 in this round
       if (tr >= total) break;
-      const int ob = __shfl_sync(TR_FULL, bv, own[k]), od = __shfl_sync(TR_FULL, dv, own[k]);
-      const int om = __shfl_sync(TR_FULL, vmax, own[k]);
+      const int ob = __shfl_sync(TR_FULL, fb, own[k]), od = __shfl_sync(TR_FULL, fd, own[k]);
+      const int om = __shfl_sync(TR_FULL, fm, own[k]);
       const int q = w[k] <= om ? find(w[k], ob, od) : -1;
       const unsigned hm = __ballot_sync(TR_FULL, q >= 0);
       if (hm == 0) continue;
       const int prior = __shfl_sync(TR_FULL, mycnt, own[k]);
-      const int64_t tbase = __shfl_sync(TR_FULL, rb, own[k]);
-      const int eo = __shfl_sync(TR_FULL, e, own[k]);
+      const int64_t tbase = __shfl_sync(TR_FULL, frb, own[k]);
       if (q >= 0) {
         const int lo = max(bo[k] - tr, 0);
         const unsigned below = hm & lt & ~((1u << lo) - 1u);
-        const int64_t euw = (int64_t)eo + 1 + (tr + lane - bo[k]);
+        const int64_t euw = (int64_t)eo[k] + 1 + (tr + lane - bo[k]);
         count_hit<kSearch>(a, nullptr, ob, q, euw, tbase + prior + __popc(below));
       }
-      if (sl > 0) {
-        const int lo = P - sl - tr, hi = P - 1 - tr;
-        if (hi >= 0 && lo <= 31) {
-          const int l0 = max(lo, 0), l1 = min(hi, 31);
-          const unsigned seg = (l1 == 31 ? 0xFFFFFFFFu : ((1u << (l1 + 1)) - 1u)) &
-                               ~((1u << l0) - 1u);
-          mycnt += __popc(hm & seg);
-        }
-      }
+      mycnt += own_hits(hm, fw.S - tr, P - tr);
     }
   }
-  if (valid && shrt) {
-    if (a.tb) a.cuv[e] = mycnt;
-    if (mycnt) atomicAdd(&a.supA[e], mycnt);
+  if (mycnt) {  // cuv starts at zero
+    if (a.tb) a.cuv[fe] = mycnt;
+    atomicAdd(&a.supA[fe], mycnt);
   }
   // long walks: the whole warp on one edge, stopping past its head's max
   unsigned lm = __ballot_sync(TR_FULL, valid && !shrt);
