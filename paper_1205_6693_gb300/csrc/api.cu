@@ -400,6 +400,8 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
     in.graphs = G;
     in.row_off = d_row_off;
     in.voff = d_voff;
+    for (int32_t i = 0; i < G; i++)
+      if (h_voff[i + 1] - h_voff[i] > in.max_n) in.max_n = h_voff[i + 1] - h_voff[i];
   }
   TR_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), s));
 

@@ -91,6 +91,7 @@ struct RowsIn {
   int32_t graphs = 1;
   const int64_t *row_off = nullptr;
   const int64_t *voff = nullptr;
+  int64_t max_n = 0;             // batch: the most vertices of one graph
 };
 
 // Small control words of one decomposition, zeroed together by build_graph:
@@ -102,8 +103,9 @@ struct ZeroBlock {
   int list_err;  // set by the list builders, reported with the peel's result
 };
 
-// Degree-ordered oriented CSR (vertices relabelled by ascending (degree, id)
-// so that an edge points from its lower-ranked to its higher-ranked end).
+// Degree-ordered oriented CSR (vertices relabelled by ascending (degree, id), in
+// a batch by (graph, degree, id) or (degree, id), so that an edge points from
+// its lower-ranked to its higher-ranked end).
 // Canonical edge id e = position in adjp.
 struct Csr {
   int64_t n = 0, m = 0, rows = 0;
@@ -112,7 +114,7 @@ struct Csr {
   int32_t *esrc = nullptr;   // [m]   tail (lower-ranked endpoint) of edge e
   int32_t *row2e = nullptr;  // [rows] row -> e, -1 for self-loop rows
   int32_t *order = nullptr;  // [n]   rank -> input vertex id
-  int32_t *sdeg = nullptr;   // [n]   degree of the vertex of each rank (ascending)
+  int32_t *sdeg = nullptr;   // [n]   degree of the vertex of each rank
   ZeroBlock *zero = nullptr; // set by build_graph
 };
 

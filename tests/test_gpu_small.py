@@ -115,3 +115,32 @@ def test_small_batch_and_bad_ids(ctx):
     with pytest.raises(T.TrussError) as ei:
         ctx.decompose_batch(ns, off, sb, d, torch.empty_like(s), torch.empty_like(s))
     assert ei.value.code == T.TRUSS_EINVAL
+
+
+@pytest.mark.parametrize("name", ["empty graphs", "one graph", "too wide to rank by graph"])
+def test_batch_ranked_by_graph_on_the_general_path(general, name):
+    # vertices ordered by (graph, degree, id), and by (degree, id) where graph
+    # number and degree do not fit one word; empty graphs at both ends
+    sizes = {"empty graphs": [0, 0, 700, 0, 1, 2, 3, 90, 0], "one graph": [500],
+             "too wide to rank by graph": [60] * 2047 + [1 << 21] + [60] * 10}[name]
+    rng = np.random.default_rng(3)
+    n = np.array(sizes, np.int64)
+    rows = np.where(n > 1, np.minimum(4 * n, 3000), 0)
+    off = np.concatenate([[0], np.cumsum(rows)]).astype(np.int64)
+    g = np.repeat(np.arange(len(n)), rows)
+    # ends drawn from the first 300 vertices: graphs dense in triangles
+    src, dst = (np.minimum((rng.random(len(g)) * np.minimum(n[g], 300)).astype(np.int32),
+                           n[g] - 1).astype(np.int32) for _ in range(2))
+    s, d = torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()
+    sup, tr = torch.full_like(s, -7), torch.full_like(s, -7)
+    kmax = torch.full((len(n),), -7, dtype=torch.int32, device="cuda")
+    general.decompose_batch(n, off, s, d, sup, tr, kmax)
+    sup, tr, kmax = sup.cpu().numpy(), tr.cpu().numpy(), kmax.cpu().numpy()
+    for i in range(len(n)):
+        a, b = off[i], off[i + 1]
+        if a == b:
+            assert kmax[i] == 0
+            continue
+        ref = oracle.truss(int(n[i]), src[a:b], dst[a:b])
+        assert np.array_equal(sup[a:b], ref.support) and np.array_equal(tr[a:b], ref.truss)
+        assert kmax[i] == ref.kmax
