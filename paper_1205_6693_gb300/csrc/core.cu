@@ -18,14 +18,16 @@
 //        a neighbour in the same frontier is simply skipped.
 //
 // Vertex state is one word, the current degree, with the top bit set once the
-// vertex is removed: a neighbour costs one read and, if alive, one decrement.
-// A vertex marked while others still decrement it only loses counts that no
-// longer matter (its degree stays >= 0: every neighbour is removed once).
+// vertex is removed.  A removed vertex takes one from the word of each of its
+// neighbours, alive or not, without reading it first: the low part of a
+// removed vertex's word is the number of its neighbours still alive, each of
+// which takes one from it once, so it never runs into the mark.
 // Neighbours come from a symmetric adjacency built from the oriented CSR.  A
 // frontier vertex is split into work items of kItem neighbours, as in the
 // edge peel, so a warp's share of a sub-round is bounded whatever the degrees.
-// Phases end as in the edge peel (phase_end).  R-MAT scale 20:
-// 5.15 -> 5.04 ms.
+// Phases end as in the edge peel (phase_end).  R-MAT scale 20: 5.15 ms with
+// phase counters read by every warp and a state read before each decrement,
+// 5.04 with the counters passed on, 4.47 now.
 #include <climits>
 
 #include "engine.h"
@@ -197,28 +199,53 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
     }
     int lmin = INT_MAX, llive = 0;  // of this lane
     bool lany = false;
-    for (int64_t base = (int64_t)gwarp * 32; base < nAlive; base += (int64_t)twarps * 32) {
-      const int64_t i = base + lane;
-      const int v = i < nAlive ? __ldcg(&alive[i]) : -1;
-      const uint32_t w = v >= 0 ? __ldcg(&a.word[v]) : kGone;
-      const bool live = (int32_t)w >= 0;
-      const bool toF = live && (int)w <= k;
-      const bool keep = live && !toF;
-      if (toF) {
-        a.word[v] = kGone | w;
-        lany = true;
-        if (w == 0) a.core[v] = k;  // no neighbour left: no item
+    // 4 x 32 entries per warp iteration, all loads before any decision
+    constexpr int kScanU = 4;
+    for (int64_t base = (int64_t)gwarp * 32 * kScanU; base < nAlive;
+         base += (int64_t)twarps * 32 * kScanU) {
+      int v[kScanU];
+      uint32_t w[kScanU];
+#pragma unroll
+      for (int u = 0; u < kScanU; u++) {
+        const int64_t i = base + u * 32 + lane;
+        v[u] = i < nAlive ? __ldcg(&alive[i]) : -1;
       }
-      push_items(a, toF && w > 0, v, wb, F, qf);
-      if (compact) push_alive(a, keep, v, wb, alive2, &scan->listed);
-      if (keep) {
-        lmin = min(lmin, (int)w);
-        llive++;
+#pragma unroll
+      for (int u = 0; u < kScanU; u++) w[u] = v[u] >= 0 ? __ldcg(&a.word[v[u]]) : kGone;
+      unsigned pend = 0;  // entries of this lane that join the frontier
+#pragma unroll
+      for (int u = 0; u < kScanU; u++) {
+        const bool live = (int32_t)w[u] >= 0;
+        const bool toF = live && (int)w[u] <= k;
+        const bool keep = live && !toF;
+        if (toF) {
+          a.word[v[u]] = kGone | w[u];
+          lany = true;
+          if (w[u] == 0) a.core[v[u]] = k;  // no neighbour left: no item
+          else pend |= 1u << u;
+        }
+        if (compact) push_alive(a, keep, v[u], wb, alive2, &scan->listed);
+        if (keep) {
+          lmin = min(lmin, (int)w[u]);
+          llive++;
+        }
+      }
+      while (__any_sync(TR_FULL, pend != 0)) {
+        int q = 0;
+        const bool has = pend != 0;
+        if (has) {
+          const int b = __ffs(pend) - 1;
+          pend &= pend - 1;
+#pragma unroll
+          for (int u = 0; u < kScanU; u++)
+            if (b == u) q = v[u];
+        }
+        push_items(a, has, q, wb, F, qf);
       }
     }
     flush_items(a, wb, F, qf);
     if (compact) flush_alive(a, wb, alive2, &scan->listed);
-    if ((int64_t)gwarp * 32 < nAlive) {
+    if ((int64_t)gwarp * 32 * kScanU < nAlive) {
       lmin = __reduce_min_sync(TR_FULL, lmin);
       llive = __reduce_add_sync(TR_FULL, llive);
       const bool wany = __any_sync(TR_FULL, lany);
@@ -282,18 +309,13 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
         for (int q = 0; q < 2; q++) {
           const int jj = j + 8 * q;
           w[q] = jj < cnt ? __ldg(&a.sadj[lb + jj]) : -1;
-        }
-#pragma unroll
-        for (int q = 0; q < 2; q++) {
           if (w[q] >= 0 && (uint32_t)w[q] >= (uint32_t)a.n) {
             raise_error(&ctl->phase[ph % 3], &ctl->err, TRUSS_ECHECK);
             w[q] = -1;
           }
-          x[q] = w[q] >= 0 ? __ldcg(&a.word[w[q]]) : kGone;
         }
 #pragma unroll
-        for (int q = 0; q < 2; q++)
-          x[q] = (int32_t)x[q] >= 0 ? atomicSub(&a.word[w[q]], 1u) : kGone;
+        for (int q = 0; q < 2; q++) x[q] = w[q] >= 0 ? atomicSub(&a.word[w[q]], 1u) : kGone;
         // one push_items site: each step pushes one pending neighbour per lane
         unsigned pend = (x[0] == (uint32_t)(k + 1) ? 1u : 0u) | (x[1] == (uint32_t)(k + 1) ? 2u : 0u);
         while (__any_sync(TR_FULL, pend != 0)) {
