@@ -26,6 +26,7 @@ struct truss_ctx {
   cudaEvent_t ev[8] = {};
   bool have_events = false;
   int sms = 0;
+  int peel_sms = 0;  // SMs the peel may use (0 = all)
 };
 
 namespace tr {
@@ -478,6 +479,7 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
     sg.mark();  // 3
     tr::PeelCfg pcfg;
     pcfg.sms = ctx->sms;
+    pcfg.max_sms = ctx->peel_sms;
     pcfg.variant = ctx->opts.peel_variant;
     pcfg.count = ctx->opts.count_bytes != 0 && !tids;
     if (ctx->opts.wait_limit_ns > 0) pcfg.wait_ns = ctx->opts.wait_limit_ns;
@@ -1040,6 +1042,9 @@ void ctx_trim(truss_ctx *ctx, size_t max_bytes) {
 }
 const truss_opts *ctx_opts(truss_ctx *ctx) { return &ctx->opts; }
 void ctx_set_limit(truss_ctx *ctx, size_t bytes) { ctx->arena.set_limit(bytes); }
+int ctx_sms(truss_ctx *ctx) { return ctx->sms; }
+// Share of the device that the context's peels take (0 = as much as suits them).
+void ctx_set_peel_sms(truss_ctx *ctx, int sms) { ctx->peel_sms = sms; }
 }  // namespace tr
 
 extern "C" {

@@ -43,6 +43,8 @@ int ctx_device(truss_ctx *ctx);
 const truss_opts *ctx_opts(truss_ctx *ctx);
 void ctx_trim(truss_ctx *ctx, size_t max_bytes);
 void ctx_set_limit(truss_ctx *ctx, size_t bytes);
+int ctx_sms(truss_ctx *ctx);
+void ctx_set_peel_sms(truss_ctx *ctx, int sms);
 }  // namespace tr
 
 namespace {
@@ -79,6 +81,7 @@ struct truss_server {
   std::vector<std::thread> workers;
   int64_t inflight_fp = 0;
   int inflight = 0;
+  int busy = 0;  // workers with a job
   bool stopping = false;
   uint64_t next_id = 1;
   // statistics
@@ -188,6 +191,7 @@ void worker_main(truss_server *S) {
   int64_t dcap = 0;
   for (;;) {
     std::vector<Request *> job;
+    int sharers = 1;  // workers that this run is likely to share the device with, and itself
     {
       std::unique_lock<std::mutex> lk(S->mu);
       S->cv_work.wait(lk, [&] {
@@ -212,8 +216,14 @@ void worker_main(truss_server *S) {
       S->inflight_fp += fp;
       S->admitted += (int64_t)job.size();
       S->launches++;
+      S->busy++;
+      sharers = (int)std::min<int64_t>(S->o.streams, S->busy + (int64_t)S->pending.size());
     }
     if (rc == TRUSS_OK) {
+      // The peel is a chain of short phases that leaves most of its SMs idle,
+      // so runs that overlap take a share each instead of one after another
+      // (24 requests of 1 K to 2 M rows: 20.2 -> 19.0 ms).
+      tr::ctx_set_peel_sms(ctx, sharers > 1 ? tr::ctx_sms(ctx) / sharers : 0);
       // workspace cap of this run: twice the projection, or the whole budget
       // for a request queued again after running out of its cap
       size_t cap = 0;
@@ -231,6 +241,7 @@ void worker_main(truss_server *S) {
     }
     {
       std::lock_guard<std::mutex> lk(S->mu);
+      S->busy--;
       for (Request *r : job) {
         S->inflight--;
         S->inflight_fp -= r->fp;
