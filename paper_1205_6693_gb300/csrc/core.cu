@@ -27,7 +27,8 @@
 // edge peel, so a warp's share of a sub-round is bounded whatever the degrees.
 // Phases end as in the edge peel (phase_end).  R-MAT scale 20: 5.15 ms with
 // phase counters read by every warp and a state read before each decrement,
-// 5.04 with the counters passed on, 4.47 now.
+// 5.04 with the counters passed on, 4.47 without the state read, 4.35 with
+// vertices staged and expanded at the flush.
 #include <climits>
 
 #include "engine.h"
@@ -39,7 +40,7 @@ namespace {
 constexpr int kBlock = 512;
 constexpr int kWarps = kBlock / 32;
 constexpr int kItem = 16;  // neighbours per work item (8 lanes x 2)
-constexpr int kWQ = 64;    // work items staged per warp
+constexpr int kWP = 32;    // pushed vertices staged per warp (one per lane)
 constexpr int kWA = 128;   // alive-list entries staged per warp
 
 struct CoreCtl : PhaseCtl {
@@ -63,24 +64,61 @@ constexpr uint32_t kGone = 0x80000000u;
 
 __device__ __forceinline__ int items_of(int len) { return len > 0 ? (len + kItem - 1) / kItem : 1; }
 
+// Per-warp staging buffers in shared memory (counts are warp-uniform).
 struct WarpBuf {
-  int4 *items;
-  int ni;
+  int32_t *push;  // vertices pushed to the next frontier, not yet expanded
+  int np;
   int32_t *alive;
   int na;
 };
 
-__device__ __forceinline__ void flush_items(const CoreArgs &a, WarpBuf &wb, int4 *Q,
-                                            unsigned long long *qctr) {
-  if (wb.ni == 0) return;
+__device__ __forceinline__ int4 make_item(int v, int64_t lb, int L, int it) {
+  const int64_t off = lb + (int64_t)it * kItem;
+  const int cnt = min(kItem, L - it * kItem);
+  return make_int4(v, max(cnt, 0) | ((it == 0) << 8), (int)(uint32_t)off,
+                   (int)(uint32_t)((uint64_t)off >> 32));
+}
+
+// Expand the staged vertices into work items and append them to queue Q with
+// one reservation; their offsets are loaded together here, not one dependent
+// round trip per push.  A single one, as most flushes have, needs no scan.
+__device__ __forceinline__ void flush_push(const CoreArgs &a, WarpBuf &wb, int4 *Q,
+                                           unsigned long long *qctr) {
+  const int np = wb.np;
+  if (np == 0) return;
   const int lane = lane_id();
-  uint32_t b = 0;
-  if (lane == 0) b = reserve_items(qctr, wb.ni);
-  const uint32_t b0 = __shfl_sync(TR_FULL, b, 0);
-  for (int t = lane; t < wb.ni; t += 32)
-    if (b0 + t < a.item_cap) Q[b0 + t] = wb.items[t];
+  const bool v = lane < np;
+  const int p = v ? wb.push[lane] : 0;
+  const int64_t lb = v ? __ldg(&a.soff[p]) : 0;
+  const int L = v ? (int)(__ldg(&a.soff[p + 1]) - lb) : 0;
+  const int n = v ? items_of(L) : 0;
+  if (np == 1) {
+    const int tot = __shfl_sync(TR_FULL, n, 0);
+    uint32_t at = 0;
+    if (lane == 0) at = reserve_items(qctr, tot);
+    at = __shfl_sync(TR_FULL, at, 0);
+    const int po = __shfl_sync(TR_FULL, p, 0), Lo = __shfl_sync(TR_FULL, L, 0);
+    const int64_t lbo = __shfl_sync(TR_FULL, lb, 0);
+    for (int it = lane; it < tot; it += 32)
+      if (at + it < a.item_cap) Q[at + it] = make_item(po, lbo, Lo, it);
+  } else {
+    const int P = warp_incl_scan(n);
+    uint32_t b = 0;
+    if (lane == 31) b = reserve_items(qctr, P);
+    const int tot = __shfl_sync(TR_FULL, P, 31);
+    const uint32_t base = __shfl_sync(TR_FULL, b, 31);
+    for (int u0 = 0; u0 < tot; u0 += 32) {
+      const int t = u0 + lane;
+      const int o = warp_owner(P, t < tot ? t : tot - 1);
+      const int po = __shfl_sync(TR_FULL, p, o), i0 = __shfl_sync(TR_FULL, P - n, o);
+      const int Lo = __shfl_sync(TR_FULL, L, o);
+      const int64_t lbo = __shfl_sync(TR_FULL, lb, o);
+      const uint32_t idx = base + t;
+      if (t < tot && idx < a.item_cap) Q[idx] = make_item(po, lbo, Lo, t - i0);
+    }
+  }
   __syncwarp();
-  wb.ni = 0;
+  wb.np = 0;
 }
 
 __device__ __forceinline__ void flush_alive(const CoreArgs &a, WarpBuf &wb, int32_t *A2,
@@ -107,53 +145,17 @@ __device__ __forceinline__ void push_alive(const CoreArgs &a, bool keep, int v, 
   wb.na += tot;
 }
 
-// Append the work items of vertex p (lanes with `push`).  All lanes call it.  Batches larger than the staging buffer go straight to Q.
+// Stage vertex p (for each lane with `push`) for expansion into work items of
+// the next frontier.  All lanes call it.
 __device__ __forceinline__ void push_items(const CoreArgs &a, bool push, int p, WarpBuf &wb,
                                            int4 *Q, unsigned long long *qctr) {
-  const int lane = lane_id();
-  int n = 0, L = 0;
-  int64_t lb = 0;
-  if (push) {
-    lb = __ldg(&a.soff[p]);
-    L = (int)(__ldg(&a.soff[p + 1]) - lb);
-    n = items_of(L);
-  }
-  const int P = warp_incl_scan(n);
-  const int tot = __shfl_sync(TR_FULL, P, 31);
-  if (tot == 0) return;
-  int4 *dst;
-  uint32_t b0;
-  if (tot > kWQ) {
-    uint32_t b = 0;
-    if (lane == 31) b = reserve_items(qctr, tot);
-    b0 = __shfl_sync(TR_FULL, b, 31);
-    dst = Q;
-  } else {
-    if (wb.ni + tot > kWQ) flush_items(a, wb, Q, qctr);
-    b0 = wb.ni;
-    dst = wb.items;
-  }
-  const uint32_t lim = tot > kWQ ? a.item_cap : (uint32_t)kWQ;
-  for (int t0 = 0; t0 < tot; t0 += 32) {
-    const int t = t0 + lane;
-    const int o = warp_owner(P, t < tot ? t : tot - 1);
-    const int po = __shfl_sync(TR_FULL, p, o);
-    const int Po = __shfl_sync(TR_FULL, P, o);
-    const int no = __shfl_sync(TR_FULL, n, o);
-    const int Lo = __shfl_sync(TR_FULL, L, o);
-    const int64_t lbo = __shfl_sync(TR_FULL, lb, o);
-    const uint32_t idx = b0 + t;
-    if (t < tot && idx < lim) {
-      const int it = t - (Po - no);
-      const int start = it * kItem;
-      const int cnt = Lo > 0 ? min(kItem, Lo - start) : 0;
-      const int64_t off = lbo + start;
-      dst[idx] = make_int4(po, cnt | ((it == 0) << 8), (int)(uint32_t)off,
-                           (int)(uint32_t)((uint64_t)off >> 32));
-    }
-  }
+  const unsigned mask = __ballot_sync(TR_FULL, push);
+  if (mask == 0) return;
+  const int tot = __popc(mask);
+  if (wb.np + tot > kWP) flush_push(a, wb, Q, qctr);
+  if (push) wb.push[wb.np + __popc(mask & ((1u << lane_id()) - 1u))] = p;
   __syncwarp();
-  if (tot <= kWQ) wb.ni += tot;
+  wb.np += tot;
 }
 
 __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
@@ -165,10 +167,10 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
   const uint32_t twarps = gridDim.x * kWarps;
   const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
   CoreCtl *ctl = a.ctl;
-  __shared__ int4 s_items[kWarps][kWQ];
+  __shared__ int32_t s_push[kWarps][kWP];
   __shared__ int32_t s_alive[kWarps][kWA];
   __shared__ int s_minres, s_live, s_any;
-  WarpBuf wb{s_items[wib], 0, s_alive[wib], 0};
+  WarpBuf wb{s_push[wib], 0, s_alive[wib], 0};
   if (threadIdx.x == 0) {
     s_minres = INT_MAX;
     s_live = 0;
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
         push_items(a, has, q, wb, F, qf);
       }
     }
-    flush_items(a, wb, F, qf);
+    flush_push(a, wb, F, qf);
     if (compact) flush_alive(a, wb, alive2, &scan->listed);
     if ((int64_t)gwarp * 32 * kScanU < nAlive) {
       lmin = __reduce_min_sync(TR_FULL, lmin);
@@ -327,7 +329,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
           push_items(a, has, q, wb, N, qn);
         }
       }
-      flush_items(a, wb, N, qn);
+      flush_push(a, wb, N, qn);
       if (!phase_end(ctl, a.wait_ns, ph, &nCur, nullptr, nullptr)) return;
       ph++;
       if (leader) ctl->subrounds++;
