@@ -67,7 +67,9 @@ typedef struct truss_ctx truss_ctx;
 typedef struct truss_opts {
   /* Upper limit, in nanoseconds, of any device-side wait (the grid-wide
    * barrier of the persistent peel kernel).  A wait that exceeds it makes the
-   * call return TRUSS_ETIMEOUT.  0 = default (4 s). */
+   * call return TRUSS_ETIMEOUT.  0 = default (4 s).  With a limit set, small
+   * graphs are built by the launches that wait for nothing instead of the one
+   * whose blocks meet at barriers (slower; same results). */
   int64_t wait_limit_ns;
   /* Non-zero: record CUDA events around each stage (build, support, triangle
    * lists, peel, scatter) so truss_last_stats reports stage times. */
@@ -81,11 +83,12 @@ typedef struct truss_opts {
    * entries are staged in shared memory, longer ones are read from global
    * memory (0 = the staging capacity, 512; larger values are clamped). */
   int32_t support_stage_max;
-  /* Peel kernel variant: 0 or 2 = two 512-thread blocks per SM, one work item
-   * per lane group; 1 = one block per SM, two items per lane group; 3 = one
-   * block per SM, one item; 4 = the barrier-free peel (a destroyed bit per
-   * triangle and a work queue per level instead of sub-rounds; it needs the
-   * triangle records and fewer than 2^32 of them, else variant 0 runs). */
+  /* Peel kernel variant: 0 or 2 = two 512-thread blocks per SM (on fewer SMs
+   * for small graphs), one work item per lane group; 1 = one block per SM,
+   * two items per lane group; 3 = one block per SM, one item; 4 = the
+   * barrier-free peel (a destroyed bit per triangle and a work queue per level
+   * instead of sub-rounds; it needs the triangle records and fewer than 2^32
+   * of them, else variant 0 runs). */
   int32_t peel_variant;
   /* Target walk cost (out-list entries) of one warp range of the support
    * walk (0 = 16384). */

@@ -639,8 +639,13 @@ int build_graph(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, Sup
   TR_CUDA(cudaMemsetAsync(out->zero, 0, sizeof(ZeroBlock), s));
   // the scans add up tiles of edge costs in 31 bits
   if (cfg.small_paths && in.rows > 0 && in.rows <= kSmallRows && in.n <= kSmallRows &&
-      walk_edge_cost(cfg) <= kSmallRows / 2)
-    return build_small(A, in, cfg, out, prep, s);
+      walk_edge_cost(cfg) <= kSmallRows / 2) {
+    const int rc = build_small(A, in, cfg, out, prep, s);
+    // its blocks could not meet in time (the device is taken by other work):
+    // the general path waits for nothing
+    if (rc != TRUSS_ETIMEOUT) return rc;
+    *prep = SupportPrep{};
+  }
   return build_csr(A, in, out, d_err, s);
 }
 

@@ -1135,10 +1135,13 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportPrep
     TR_TRY(launch_walk_v(A, a, cfg, s));
   }
   int64_t total = 0;
-  if (pre.valid) {
-    TR_TRY(small_offsets(A, g, pre, recs ? cuv : nullptr, cfg.sms, sup, toff, &total, &out->small,
-                         s));
-  } else {
+  int done = TRUSS_ETIMEOUT;  // small graphs: in one launch, unless its blocks cannot meet in time
+  if (pre.valid)
+    done = small_offsets(A, g, pre, recs ? cuv : nullptr, cfg.sms, sup, toff, &total, &out->small,
+                         s);
+  if (done != TRUSS_OK) {
+    if (done != TRUSS_ETIMEOUT) return done;
+    out->small = SmallLists{};
     int64_t *sup64 = A.get<int64_t>(m + 1);
     if (!sup64) return TRUSS_ENOMEM;
     k_sum<<<grid_for(m + 1, 256, 152 * 16), 256, 0, s>>>(m, pre.supA, pre.supB, sup, sup64);
