@@ -531,7 +531,7 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
     if (want_truss) {
       st.design_bytes_peel = (so.in_place ? 40.0 : 28.0) * (double)g.m +
                              16.0 * (double)pr.entries + 8.0 * (double)pr.decrements +
-                             16.0 * (double)pr.scanned;
+                             12.0 * (double)pr.scanned;
       const double smin = (double)pr.sum_min_alive;
       st.bytes_peel = 12.0 * smin + 12.0 * (smin - (double)g.m) + 8.0 * (double)g.m +
                       16.0 * (double)st.triangles + 8.0 * (double)pr.alive_levels;

@@ -493,7 +493,12 @@ __global__ void __launch_bounds__(kPeelBlock, MINB) k_peel(PeelArgs a) {
       ctl->kmax = k;
     }
     if (nCur == 0) {
-      // nothing removed had a triangle left, so the residuals stand
+      // nothing removed had a triangle left, so the residuals stand; what went
+      // counts as one sub-round
+      if (any) {
+        s++;
+        if (leader) ctl->subrounds++;
+      }
       if (live == 0) break;
       k = minres + 2;  // every alive edge has res >= k-1: skip empty levels
       continue;
