@@ -97,17 +97,17 @@ __global__ void __launch_bounds__(kBlk) k_hindex_block(const int32_t *big,
     const int64_t ob = offp[w], ib = inoff[w];
     const int dout = (int)(offp[w + 1] - ob), din = (int)(inoff[w + 1] - ib);
     const int d = dout + din;
-    // supports are clipped to d; h lies in [lo, lo + kBins << sh), and `above`
-    // supports lie beyond that
+    // supports are clipped to d; h lies in [lo, hi), and `above` supports lie
+    // beyond that
     int lo = 0, above = 0;
     int sh = 0;
     while (((int64_t)kBins << sh) < (int64_t)d + 1) sh++;
+    int64_t hi = (int64_t)kBins << sh;
     for (;; sh = sh > 11 ? sh - 11 : 0) {
       static_assert(kBins == 1 << 11, "a pass narrows the range by 11 bits");
       for (int i = threadIdx.x; i < kBins; i += kBlk) s_bin[i] = 0;
       if (threadIdx.x == 0) s_best = 0;
       __syncthreads();
-      const int64_t hi = lo + ((int64_t)kBins << sh);
       for (int i = threadIdx.x; i < d; i += kBlk) {
         const int v = min(i < dout ? __ldg(&sup[ob + i]) : __ldg(&sup[__ldg(&inedge[ib + i - dout])]), d);
         if (v >= lo && v < hi) atomicAdd(&s_bin[(v - lo) >> sh], 1);
@@ -143,9 +143,13 @@ __global__ void __launch_bounds__(kBlk) k_hindex_block(const int32_t *big,
         s_above = beyond;
       }
       __syncthreads();
+      // the next pass counts one bin of this one: the supports past it are in
+      // `above` already
       lo += s_best << sh;
+      hi = lo + ((int64_t)1 << sh);
       above = s_above;
       if (sh == 0) break;
+      __syncthreads();  // s_best is cleared by the next pass
     }
     if (threadIdx.x == 0) {
       h[w] = lo;

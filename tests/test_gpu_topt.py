@@ -188,3 +188,18 @@ def test_top_rejects_bad_ids(ctx):
     with pytest.raises(T.TrussError) as ei:
         ctx.top(5, src, dst, 1, out)
     assert ei.value.code == T.TRUSS_EINVAL
+
+
+# A hub's h-index is found by counting its supports in 2,048 bins: one pass up
+# to degree 2,047, then two.
+@pytest.mark.parametrize("deg,scale", [(2047, 11), (2048, 11), (2500, 11), (5000, 12)])
+def test_psi_of_hubs(ctx, deg, scale):
+    s, d = graphgen.rmat_raw(scale, 6 << scale, seed=deg)
+    keep = (s < deg) & (d < deg)
+    hub = np.arange(1, deg + 1, dtype=np.int32)  # vertex 0 meets all the others
+    src = np.concatenate([s[keep] + 1, np.zeros(deg, np.int32)]).astype(np.int32)
+    dst = np.concatenate([d[keep] + 1, hub]).astype(np.int32)
+    osup, ops = oracle.psi(deg + 1, src, dst)
+    for _ in range(3):
+        sup, ps = gpu_psi(ctx, deg + 1, src, dst)
+        assert np.array_equal(sup, osup) and np.array_equal(ps, ops)
