@@ -441,21 +441,23 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
 
   int32_t *truss_e = nullptr;
   tr::PeelResult pr;
-  // the per-row outputs, enqueued behind the kernels that compute them; they
-  // are written once, by the scatter: pinned host outputs in place
-  auto emit = [&]() -> int {
-    sg.mark();  // 4 (or 3 for support only: the scatter ends at the next)
-    OutBuf os, ot;
+  // The per-row outputs are enqueued behind the kernels that compute them and
+  // written once, by the scatter: pinned host outputs in place.  Their buffers
+  // are taken first, so that a call short of memory fails before its peel, the
+  // longest kernel, is launched.
+  const bool batch_k = (G > 1 || h_row_off) && kmax_out && want_truss;
+  OutBuf os, ot, ok;
+  auto stage_outputs = [&]() -> int {
     TR_TRY(stage_out(A, support_out, rows, &os, true));
     TR_TRY(stage_out(A, want_truss ? truss_out : nullptr, rows, &ot, true));
+    return stage_out(A, batch_k ? kmax_out : nullptr, G, &ok);
+  };
+  auto emit = [&]() -> int {
+    sg.mark();  // 4 (or 3 for support only: the scatter ends at the next)
     TR_TRY(tr::scatter_rows_packed(A, g, so.sup, truss_e, os.dev, ot.dev, s));
-    if (G > 1 || h_row_off) {
-      if (kmax_out && want_truss) {
-        OutBuf ok;
-        TR_TRY(stage_out(A, kmax_out, G, &ok));
-        TR_TRY(tr::batch_kmax(G, d_row_off, ot.dev, ok.dev, s));
-        TR_TRY(copy_back(ok, G, s));
-      }
+    if (batch_k) {
+      TR_TRY(tr::batch_kmax(G, d_row_off, ot.dev, ok.dev, s));
+      TR_TRY(copy_back(ok, G, s));
     }
     TR_TRY(copy_back(os, rows, s));
     TR_TRY(copy_back(ot, rows, s));
@@ -483,6 +485,7 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
     pcfg.variant = ctx->opts.peel_variant;
     pcfg.count = ctx->opts.count_bytes != 0 && !tids;
     if (ctx->opts.wait_limit_ns > 0) pcfg.wait_ns = ctx->opts.wait_limit_ns;
+    TR_TRY(stage_outputs());
     pcfg.then = emit;
     int rc = tids ? tr::run_peel_async(A, g, so, pairs, tids, so.records, pcfg, truss_e, &pr, s)
                   : tr::run_peel(A, g, so, lists, pcfg, truss_e, &pr, s);
@@ -494,6 +497,7 @@ int run_pipeline(truss_ctx *ctx, int64_t n_total, int64_t rows, const int32_t *s
     st.peel_decrements = (int64_t)pr.decrements;
     st.peel_scanned = (int64_t)pr.scanned;
   } else {
+    TR_TRY(stage_outputs());
     TR_TRY(emit());
   }
   int32_t k_host = pr.kmax;
@@ -1010,6 +1014,15 @@ int run_core_numbers(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src
   return TRUSS_OK;
 }
 
+// A failed call may have kernels and copies in flight that use the context's
+// workspace and the caller's buffers.  It returns once they have ended, as a
+// call that succeeds does: the caller may free its buffers, and the next call
+// starts over with the workspace, on any stream.
+int settled(int rc, cudaStream_t s) {
+  if (rc != TRUSS_OK && cudaStreamSynchronize(s) != cudaSuccess) cudaGetLastError();
+  return rc;
+}
+
 }  // namespace
 
 namespace tr {
@@ -1029,8 +1042,9 @@ int decompose_batch_counts(truss_ctx *ctx, int32_t G, const int64_t *n, const in
     }
     return TRUSS_OK;
   }
-  return run_pipeline(ctx, voff[G], rows, src, dst, G, row_off, voff.data(), support_out,
-                      truss_out, kmax_out, true, s, graph_m, graph_tri);
+  return settled(run_pipeline(ctx, voff[G], rows, src, dst, G, row_off, voff.data(), support_out,
+                              truss_out, kmax_out, true, s, graph_m, graph_tri),
+                 s);
 }
 int ctx_device(truss_ctx *ctx) { return ctx->device; }
 // Release the context's workspace if it holds more than max_bytes.
@@ -1112,8 +1126,10 @@ int truss_support(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src, c
                   int32_t *support_out, void *cuda_stream) {
   TR_TRY(check_common(ctx, n, rows, src, dst));
   if (rows > 0 && !support_out) return TRUSS_EINVAL;
-  return run_pipeline(ctx, n, rows, src, dst, 1, nullptr, nullptr, support_out, nullptr, nullptr,
-                      false, (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  return settled(run_pipeline(ctx, n, rows, src, dst, 1, nullptr, nullptr, support_out, nullptr,
+                              nullptr, false, s),
+                 s);
 }
 
 int truss_decompose(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src,
@@ -1121,8 +1137,10 @@ int truss_decompose(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src,
                     int32_t *kmax_out, void *cuda_stream) {
   TR_TRY(check_common(ctx, n, rows, src, dst));
   if (rows > 0 && !truss_out) return TRUSS_EINVAL;
-  return run_pipeline(ctx, n, rows, src, dst, 1, nullptr, nullptr, support_out, truss_out,
-                      kmax_out, true, (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  return settled(run_pipeline(ctx, n, rows, src, dst, 1, nullptr, nullptr, support_out, truss_out,
+                              kmax_out, true, s),
+                 s);
 }
 
 int truss_upper_bound(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src,
@@ -1130,15 +1148,16 @@ int truss_upper_bound(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *sr
                       void *cuda_stream) {
   TR_TRY(check_common(ctx, n, rows, src, dst));
   if (rows > 0 && !psi_out) return TRUSS_EINVAL;
-  return run_upper_bound(ctx, n, rows, src, dst, support_out, psi_out,
-                         (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  return settled(run_upper_bound(ctx, n, rows, src, dst, support_out, psi_out, s), s);
 }
 
 int truss_top(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src, const int32_t *dst,
               int32_t t, int32_t *truss_out, int32_t *kmax_out, void *cuda_stream) {
   TR_TRY(check_common(ctx, n, rows, src, dst));
   if (t < 1 || (rows > 0 && !truss_out)) return TRUSS_EINVAL;
-  return run_top(ctx, n, rows, src, dst, t, truss_out, kmax_out, (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  return settled(run_top(ctx, n, rows, src, dst, t, truss_out, kmax_out, s), s);
 }
 
 int truss_decompose_budget(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src,
@@ -1146,16 +1165,18 @@ int truss_decompose_budget(truss_ctx *ctx, int64_t n, int64_t rows, const int32_
                            int32_t *truss_out, int32_t *kmax_out, void *cuda_stream) {
   TR_TRY(check_common(ctx, n, rows, src, dst));
   if (budget_edges < 1 || (rows > 0 && !truss_out)) return TRUSS_EINVAL;
-  return run_bottom_up(ctx, n, rows, src, dst, budget_edges, support_out, truss_out, kmax_out,
-                       (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  return settled(run_bottom_up(ctx, n, rows, src, dst, budget_edges, support_out, truss_out,
+                               kmax_out, s),
+                 s);
 }
 
 int truss_core(truss_ctx *ctx, int64_t n, int64_t rows, const int32_t *src, const int32_t *dst,
                int32_t *core_out, int32_t *kmax_out, void *cuda_stream) {
   TR_TRY(check_common(ctx, n, rows, src, dst));
   if (n > 0 && !core_out) return TRUSS_EINVAL;
-  return run_core_numbers(ctx, n, rows, src, dst, core_out, kmax_out,
-                          (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  return settled(run_core_numbers(ctx, n, rows, src, dst, core_out, kmax_out, s), s);
 }
 
 int truss_decompose_batch(truss_ctx *ctx, int32_t G, const int64_t *n, const int64_t *row_off,
@@ -1184,8 +1205,10 @@ int truss_decompose_batch(truss_ctx *ctx, int32_t G, const int64_t *n, const int
     }
     return TRUSS_OK;
   }
-  return run_pipeline(ctx, ntot, rows, src, dst, G, row_off, voff.data(), support_out, truss_out,
-                      kmax_out, true, (cudaStream_t)cuda_stream);
+  const cudaStream_t s = (cudaStream_t)cuda_stream;
+  return settled(run_pipeline(ctx, ntot, rows, src, dst, G, row_off, voff.data(), support_out,
+                              truss_out, kmax_out, true, s),
+                 s);
 }
 
 int truss_last_stats(truss_ctx *ctx, truss_run_stats *out) {

@@ -153,6 +153,8 @@ void run_job(truss_ctx *ctx, cudaStream_t st, std::vector<Request *> &job, int32
     if (rc == TRUSS_OK)
       rc = tr::decompose_batch_counts(ctx, G, ns.data(), off.data(), *dsrc, *ddst, hs.data(),
                                       ht.data(), kmax.data(), st, gm.data(), gt.data());
+    else if (cudaStreamSynchronize(st) != cudaSuccess)  // copies of the requests' rows in flight
+      cudaGetLastError();
     for (int32_t g = 0; g < G; g++) {
       Request *r = job[g];
       r->rc = rc;

@@ -1,0 +1,52 @@
+"""Calls that fail on the device side: nothing of theirs is left running when
+they return, and the context works afterwards."""
+import numpy as np
+import pytest
+
+import graphgen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def test_call_without_room_for_its_outputs_returns_after_its_work():
+    # Outputs in pageable host memory are staged on the device.  With the whole
+    # device taken, the context's workspace (sized by earlier calls with device
+    # outputs) has no room for them: the call fails, and by then the stream is
+    # idle, so the next call may use the workspace on another stream at once.
+    from paper_1205_6693_gb300 import truss as T
+    n, rows = 1 << 18, 1 << 22
+    s, d = graphgen.rmat_raw_cuda(18, rows, seed=21)
+    sup, tr = torch.empty_like(s), torch.empty_like(s)
+    ref_sup, ref_tr = torch.empty_like(s), torch.empty_like(s)
+    h_sup, h_tr = np.empty(rows, np.int32), np.empty(rows, np.int32)
+    # lists from a second walk: the working set does not depend on what is free
+    warm = T.Context(0, lists_by_walk=1)  # loads every kernel of the call
+    warm.decompose(n, s, d, h_sup, h_tr)
+    warm.close()
+    ctx = T.Context(0, lists_by_walk=1)
+    hold = []
+    try:
+        for _ in range(2):
+            ctx.decompose(n, s, d, ref_sup, ref_tr)
+        other = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        size = 1 << 37
+        while size >= 8 << 20:  # the workspace grows by 64 MB or more
+            try:
+                hold.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.OutOfMemoryError:
+                size //= 2
+        with pytest.raises(T.TrussError) as ei:
+            ctx.decompose(n, s, d, h_sup, h_tr)
+        idle = torch.cuda.current_stream().query()
+        assert ei.value.code == T.TRUSS_ENOMEM
+        assert idle
+        ctx.decompose(n, s, d, sup, tr, stream=other.cuda_stream)
+        hold.clear()
+        torch.cuda.empty_cache()
+        assert torch.equal(sup, ref_sup) and torch.equal(tr, ref_tr)
+    finally:
+        hold.clear()
+        ctx.close()
+        torch.cuda.empty_cache()
