@@ -356,7 +356,7 @@ typedef struct truss_serve_stats {
  * supports and peel queues, 16 per vertex, and 8-byte triangle-list entries
  * for an assumed 3 x 32 triangle incidences per row (the exact figure is
  * known only after the support pass).  A run's workspace is capped at twice
- * the projection of its requests; a request that needs more (a graph much
+ * the projection of its requests and 256 KB; a request that needs more (a graph much
  * denser in triangles than assumed) fails that run with TRUSS_ENOMEM, is
  * queued again once at the head of the queue with the whole budget as its
  * footprint, and then runs alone with the whole budget as its cap: it

@@ -153,15 +153,26 @@ struct ListRanges {
 };
 constexpr int kListEdgeCost = 4;  // range cost per edge (next to its records)
 constexpr int kListCounters = 16384;  // shared cursor counters per range (64 KB)
+// A range's out-edges should fit the counters.  Ranges of that size leave
+// most blocks idle on small graphs: those take four ranges per block, but
+// none under kListMinCost (list passes of the 4,096-vertex graph 62 -> 25 us; of
+// R-MAT scale 15 the same 165 us).
+constexpr int64_t kListMaxCost = (int64_t)kListCounters * kListEdgeCost / 2, kListMinCost = 512;
+constexpr int kListFit = 4 * 2 * 152;
 __host__ __device__ inline ListRanges list_ranges(int64_t triangles, int64_t m) {
-  // A range's out-edges should fit the counters.  Ranges of that size leave
-  // most blocks idle on small graphs: those take four ranges per block, but
-  // none under kMin (list passes of the 4,096-vertex graph 62 -> 25 us; of
-  // R-MAT scale 15 the same 165 us).
-  constexpr int64_t kMax = (int64_t)kListCounters * kListEdgeCost / 2, kMin = 512;
-  const int64_t total = triangles + 2 * kListEdgeCost * m, fit = total / (4 * 2 * 152);
-  const int64_t cost = fit > kMax ? kMax : fit < kMin ? kMin : fit;
+  const int64_t total = triangles + 2 * kListEdgeCost * m, fit = total / kListFit;
+  const int64_t cost = fit > kListMaxCost ? kListMaxCost : fit < kListMinCost ? kListMinCost : fit;
   return {cost, (triangles + kListEdgeCost * m) / cost + 1, total / cost + 1};
+}
+// The most ranges that list_ranges gives any number of triangles up to `most`:
+// no range costs less than kListMinCost, and a range of total / kListFit,
+// rounded down from at least kListMinCost, loses less than one part in that.
+inline int64_t list_ranges_most(int64_t most, int64_t m) {
+  const int64_t total = most + 2 * kListEdgeCost * m;
+  const int64_t fitted = kListFit + kListFit / kListMinCost + 2;
+  const int64_t widest = total / kListMaxCost + 1 > fitted ? total / kListMaxCost + 1 : fitted;
+  const int64_t narrow = total / kListMinCost + 1;
+  return narrow < widest ? narrow : widest;
 }
 
 // What a small graph's build leaves ready for the support walk (small.cu).

@@ -177,6 +177,11 @@ void run_job(truss_ctx *ctx, cudaStream_t st, std::vector<Request *> &job, int32
   }
 }
 
+// Workspace of a run beside its share per row and vertex: control words, the
+// smallest tables, and arrays rounded up to the arena's 256 bytes (a request of
+// one row takes 22 KB, of 100 rows 40 KB; the device gives 64 MB at a time).
+constexpr size_t kRunFixed = 256 << 10;
+
 // True if request r can be admitted now.
 bool fits(const truss_server *S, const Request *r, int extra_count, int64_t extra_fp) {
   if (S->inflight + extra_count + 1 > S->o.max_inflight) return false;
@@ -228,7 +233,7 @@ void worker_main(truss_server *S) {
       tr::ctx_set_peel_sms(ctx, sharers > 1 ? tr::ctx_sms(ctx) / sharers : 0);
       // workspace cap of this run: twice the projection, or the whole budget
       // for a request queued again after running out of its cap
-      size_t cap = 0;
+      size_t cap = job[0]->retried ? 0 : kRunFixed;
       for (Request *r : job) cap += (size_t)(r->retried ? r->fp : 2 * r->fp);
       tr::ctx_set_limit(ctx, cap);
       run_job(ctx, st, job, &dsrc, &ddst, &dcap);

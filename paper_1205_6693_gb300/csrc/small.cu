@@ -511,19 +511,26 @@ __global__ void __launch_bounds__(kBlock, 2) k_small_offsets(OffsetArgs a) {
 constexpr int64_t kSmallRows = 5 << 19;
 constexpr int64_t kWaitNs = 4000000000LL;
 
-// Blocks of a cooperative launch of `kern` for about `work` elements: one per
-// SM, fewer for small graphs (two elements per thread), never more than fit.
-template <class Args>
-int launch_small(void (*kern)(Args), int64_t work, int sms, Args a, int64_t *(Args::*part),
-                 int per_block, Arena &A, cudaStream_t s) {
-  int occ = 0;
-  TR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kBlock, 0));
-  if (occ < 1) return TRUSS_ECUDA;
+// Blocks of a cooperative launch for about `work` elements: one per SM, fewer
+// for small graphs (two elements per thread).
+int small_grid(int64_t work, int sms, int *out) {
+  if (sms <= 0) {
+    int dev = 0;
+    TR_CUDA(cudaGetDevice(&dev));
+    TR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  }
   int64_t grid = (work + 2 * kBlock - 1) / (2 * kBlock);
   if (grid > sms) grid = sms;
   if (grid < 8) grid = sms < 8 ? sms : 8;
-  a.*part = A.get<int64_t>(per_block * grid);
-  if (!(a.*part)) return TRUSS_ENOMEM;
+  *out = (int)grid;
+  return TRUSS_OK;
+}
+
+template <class Args>
+int launch_small(void (*kern)(Args), int grid, Args a, cudaStream_t s) {
+  int occ = 0;
+  TR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kBlock, 0));
+  if (occ < 1) return TRUSS_ECUDA;
   void *args[] = {&a};
   TR_CUDA(cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)grid), dim3(kBlock), args,
                                       0, s));
@@ -531,21 +538,15 @@ int launch_small(void (*kern)(Args), int64_t work, int sms, Args a, int64_t *(Ar
   return TRUSS_OK;
 }
 
-int device_sms(int sms, int *out) {
-  int dev = 0;
-  if (sms <= 0) {
-    TR_CUDA(cudaGetDevice(&dev));
-    TR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  *out = sms;
-  return TRUSS_OK;
-}
-
 int build_small(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, SupportPrep *prep,
                 cudaStream_t s) {
   const int64_t rows = in.rows, n = in.n;
-  int64_t slots = 1024;
+  // sized to the graph throughout: a run of the server has little more than
+  // the rows' share of the workspace
+  int64_t slots = 64;
   while (slots < 2 * rows) slots *= 2;
+  int grid = 0;
+  TR_TRY(small_grid(rows > n ? rows : n, cfg.sms, &grid));
   SmallArgs a{};
   a.in = in;
   a.wait_ns = kWaitNs;
@@ -559,7 +560,8 @@ int build_small(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, Sup
   a.eu = A.get<int32_t>(rows);
   a.ev = A.get<int32_t>(rows);
   a.deg = A.get<int32_t>(n);
-  a.hist = A.get<int32_t>((int64_t)kLow * (cfg.sms > 0 ? cfg.sms : 1024));
+  a.part = A.get<int64_t>(2 * (int64_t)grid);
+  a.hist = A.get<int32_t>((int64_t)kLow * grid);
   a.high = A.get<int2>(2 * rows / kLow + 1);
   a.outc = A.get<int32_t>(n);
   a.curo = A.get<int32_t>(n);
@@ -586,7 +588,8 @@ int build_small(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, Sup
   a.supB = A.get<int32_t>(rows);
   a.cuv = cfg.records ? A.get<int32_t>(rows) : nullptr;
   a.rb = A.get<int64_t>(rows + 2);
-  if (!a.keys || !a.slot_id || !a.row_slot || !a.eu || !a.ev || !a.deg || !a.hist || !a.high ||
+  if (!a.keys || !a.slot_id || !a.row_slot || !a.eu || !a.ev || !a.deg || !a.part || !a.hist ||
+      !a.high ||
       !a.outc || !a.curo || !a.curi || !a.lt || !a.lh || !a.lid || !a.newid || !a.lex2e ||
       !a.sdeg || !a.order || !a.offp || !a.inoff || !a.adjp || !a.esrc || !a.row2e || !a.inedge ||
       !a.ihead || !a.wcost || !a.bound || !a.wpre || !a.tbpre || !a.supA || !a.supB || !a.rb ||
@@ -595,9 +598,7 @@ int build_small(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, Sup
   a.ecost = walk_edge_cost(cfg);
   a.range_work = walk_range_work(cfg);
   TR_TRY(walk_warps(cfg, &a.warps));
-  int sms = 0;
-  TR_TRY(device_sms(cfg.sms, &sms));
-  TR_TRY(launch_small(k_small_build, rows > n ? rows : n, sms, a, &SmallArgs::part, 2, A, s));
+  TR_TRY(launch_small(k_small_build, grid, a, s));
   SmallCtl h{};
   TR_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
   TR_CUDA(cudaStreamSynchronize(s));
@@ -640,10 +641,14 @@ int build_graph(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, Sup
   // the scans add up tiles of edge costs in 31 bits
   if (cfg.small_paths && in.rows > 0 && in.rows <= kSmallRows && in.n <= kSmallRows &&
       walk_edge_cost(cfg) <= kSmallRows / 2) {
+    const std::vector<size_t> mk = A.mark();
     const int rc = build_small(A, in, cfg, out, prep, s);
-    // its blocks could not meet in time (the device is taken by other work):
-    // the general path waits for nothing
-    if (rc != TRUSS_ETIMEOUT) return rc;
+    // its blocks could not meet in time (the device is taken by other work), or
+    // its arrays, sized by rows where the general path's shrink to the distinct
+    // edges, do not fit: the general path waits for nothing and starts over
+    // with the workspace
+    if (rc != TRUSS_ETIMEOUT && rc != TRUSS_ENOMEM) return rc;
+    A.rewind(mk);
     *prep = SupportPrep{};
   }
   return build_csr(A, in, out, d_err, s);
@@ -667,9 +672,7 @@ int small_offsets(Arena &A, const Csr &g, const SupportPrep &prep, const int32_t
   a.sup = sup;
   a.toff = toff;
   if (cuv) {
-    // at most as many triangles as record slots
-    const ListRanges most = list_ranges(prep.R, m);
-    const int64_t cap = (most.n1 > most.n2 ? most.n1 : most.n2) + 4 * 2 * 152 + 2;
+    const int64_t cap = list_ranges_most(prep.R, m) + 1;  // at most as many triangles as slots
     a.cur = A.get<unsigned long long>(m);
     a.p1 = A.get<int64_t>(m + 1);
     a.p2 = A.get<int64_t>(m + 1);
@@ -682,8 +685,11 @@ int small_offsets(Arena &A, const Csr &g, const SupportPrep &prep, const int32_t
     lists->vb1 = a.vb1;
     lists->vb2 = a.vb2;
   }
-  TR_TRY(device_sms(sms, &sms));
-  TR_TRY(launch_small(k_small_offsets, m > n ? m : n, sms, a, &OffsetArgs::part, 3, A, s));
+  int grid = 0;
+  TR_TRY(small_grid(m > n ? m : n, sms, &grid));
+  a.part = A.get<int64_t>(3 * (int64_t)grid);
+  if (!a.part) return TRUSS_ENOMEM;
+  TR_TRY(launch_small(k_small_offsets, grid, a, s));
   OffsetCtl h{};
   TR_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
   TR_CUDA(cudaStreamSynchronize(s));

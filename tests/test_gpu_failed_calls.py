@@ -1,5 +1,5 @@
-"""Calls that fail on the device side: nothing of theirs is left running when
-they return, and the context works afterwards."""
+"""Calls short of device memory: one that fails leaves nothing running and its
+context usable, and one that fits by the general path takes it."""
 import numpy as np
 import pytest
 
@@ -7,6 +7,15 @@ import graphgen
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+
+def take_device(hold):
+    size = 1 << 37
+    while size >= 8 << 20:  # the workspace grows by 64 MB or more
+        try:
+            hold.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+        except torch.OutOfMemoryError:
+            size //= 2
 
 
 def test_call_without_room_for_its_outputs_returns_after_its_work():
@@ -31,18 +40,45 @@ def test_call_without_room_for_its_outputs_returns_after_its_work():
             ctx.decompose(n, s, d, ref_sup, ref_tr)
         other = torch.cuda.Stream()
         torch.cuda.synchronize()
-        size = 1 << 37
-        while size >= 8 << 20:  # the workspace grows by 64 MB or more
-            try:
-                hold.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
-            except torch.OutOfMemoryError:
-                size //= 2
+        take_device(hold)
         with pytest.raises(T.TrussError) as ei:
             ctx.decompose(n, s, d, h_sup, h_tr)
         idle = torch.cuda.current_stream().query()
         assert ei.value.code == T.TRUSS_ENOMEM
         assert idle
         ctx.decompose(n, s, d, sup, tr, stream=other.cuda_stream)
+        hold.clear()
+        torch.cuda.empty_cache()
+        assert torch.equal(sup, ref_sup) and torch.equal(tr, ref_tr)
+    finally:
+        hold.clear()
+        ctx.close()
+        torch.cuda.empty_cache()
+
+
+def test_small_graph_of_many_duplicates_fits_the_general_paths_workspace():
+    # The one-launch build holds arrays for every row, the general path for
+    # every distinct edge: with the device taken and a workspace sized by the
+    # general path (which a wait limit selects) the call still succeeds.
+    from paper_1205_6693_gb300 import truss as T
+    n, rows = 3000, 2_600_000
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    s, d = (torch.randint(0, n, (2600,), dtype=torch.int32, generator=gen,
+                          device="cuda").repeat(rows // 2600) for _ in range(2))
+    ref_sup, ref_tr = torch.empty_like(s), torch.empty_like(s)
+    sup, tr = torch.empty_like(s), torch.empty_like(s)
+    warm = T.Context(0)  # loads the kernels of the one-launch build
+    warm.decompose(n, s, d, sup, tr)
+    warm.close()
+    ctx = T.Context(0, wait_limit_ns=4_000_000_000)
+    hold = []
+    try:
+        for _ in range(2):
+            k = ctx.decompose(n, s, d, ref_sup, ref_tr)
+        torch.cuda.synchronize()
+        take_device(hold)
+        ctx.set_opts()
+        assert ctx.decompose(n, s, d, sup, tr) == k
         hold.clear()
         torch.cuda.empty_cache()
         assert torch.equal(sup, ref_sup) and torch.equal(tr, ref_tr)

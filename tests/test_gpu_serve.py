@@ -180,3 +180,25 @@ def test_dense_request_completes_or_fails_alone(T):
     # K_300 exceeds twice its projection: its first run fails and it is run
     # again alone with the whole budget, which it fits
     assert outcomes[10] == "ok" and stats["retried"] >= 1
+
+
+@pytest.mark.parametrize("max_batch", [1, 2, 64])
+def test_smallest_requests_fit_their_cap(T, max_batch):
+    # 1 to 130 rows, alone and batched: the workspace that does not shrink with
+    # the graph is not charged to the rows, so no run is repeated
+    ctx = T.truss_ctx_create(0)
+    srv = T.truss_serve_start(ctx, _serve_opts(T, streams=2, max_batch=max_batch))
+    T.truss_ctx_destroy(ctx)
+    rng = np.random.default_rng(max_batch)
+    reqs = []
+    for rows in [*range(1, 20), 31, 32, 33, 50, 64, 100, 127, 128, 129, 130]:
+        n = max(2, rows // 2)
+        reqs.append((n, *(rng.integers(0, n, rows).astype(np.int32) for _ in range(2))))
+    tickets = [T.truss_serve_submit(srv, *r) for r in reqs]
+    for (n, s, d), t in zip(reqs, tickets):
+        sup, tr = np.empty(len(s), np.int32), np.empty(len(s), np.int32)
+        T.truss_serve_wait(srv, t, -1, sup, tr)
+        ref = oracle.truss(n, s, d)
+        assert np.array_equal(sup, ref.support) and np.array_equal(tr, ref.truss)
+    stats = T.truss_serve_stop(srv)
+    assert stats["completed"] == len(reqs) and stats["retried"] == 0
