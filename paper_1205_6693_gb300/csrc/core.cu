@@ -283,7 +283,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_core(CoreArgs a) {
       ctl->kmax = k;
     }
     if (nCur == 0) {
-      // nothing removed had a neighbour left, so the degrees stand
+      // nothing removed had a neighbour left, so the degrees stand; what went
+      // counts as one sub-round
+      if (found.any && leader) ctl->subrounds++;
       if (found.live == 0) break;
       k = found.minres;  // every alive vertex has degree >= k+1: skip empty levels
       continue;

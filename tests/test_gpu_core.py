@@ -106,3 +106,24 @@ def test_core_empty_and_invalid(ctx):
         ctx.core(3, np.array([0, 5], np.int32), np.array([1, 2], np.int32),
                  np.empty(3, np.int32))
     assert ei.value.code == T.TRUSS_EINVAL
+
+
+@pytest.mark.parametrize("n,edges", [
+    (4, []),                                                    # vertices without edges only
+    (9, [(0, 1), (1, 2), (0, 2)]),                              # and a triangle
+    (12, [(0, i) for i in range(1, 7)] + [(7, 8), (8, 9)]),     # a star, a path, two without
+    (5, [(i, i + 1) for i in range(4)]),                        # none without edges
+])
+def test_every_frontier_counts_as_a_sub_round(ctx, n, edges):
+    # a frontier is what is removed together: the vertices without edges too
+    adj = [{b for e in edges for b in e if v in e and b != v} for v in range(n)]
+    alive, levels, subrounds = set(range(n)), 0, 0
+    while alive:
+        k = min(len(adj[v] & alive) for v in alive)
+        levels += 1
+        while f := {v for v in alive if len(adj[v] & alive) <= k}:
+            alive -= f
+            subrounds += 1
+    gpu_core(ctx, n, *rows_of(edges or [(0, 0)]))
+    st = ctx.stats()
+    assert (st["levels"], st["subrounds"]) == (levels, subrounds)
