@@ -22,6 +22,7 @@
 // 2 M 1.80 / 1.71, 4 M 3.00 / 3.41.  Above kSmallRows rows the table and the
 // lists leave L2, and the sorts, which stream, are faster.
 #include <climits>
+#include <cstdlib>
 
 #include "engine.h"
 
@@ -171,6 +172,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_small_build(SmallArgs a) {
   const int64_t tid = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   const int64_t nt = (int64_t)gridDim.x * kBlock;
   auto sync = [&]() { return grid_barrier(&ctl->bar, &ctl->err, a.wait_ns); };
+  if (a.wait_ns < 0 && tid == 0) raise_error(&ctl->bar, &ctl->err, TRUSS_ETIMEOUT);
   // 0. clear
   {
     ulonglong2 *k2 = (ulonglong2 *)a.keys;
@@ -470,6 +472,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_small_offsets(OffsetArgs a) {
   OffsetCtl *ctl = a.ctl;
   const int64_t tid = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   const int64_t nt = (int64_t)gridDim.x * kBlock, m = a.m, n = a.n;
+  if (a.wait_ns < 0 && tid == 0) raise_error(&ctl->bar, &ctl->err, TRUSS_ETIMEOUT);
   int64_t tot[3];
   if (!grid_scan<3>(
           &ctl->bar, &ctl->err, a.wait_ns, m, a.part, tot,
@@ -509,7 +512,15 @@ __global__ void __launch_bounds__(kBlock, 2) k_small_offsets(OffsetArgs a) {
 
 // Rows and vertices up to which the small paths are taken (see the top).
 constexpr int64_t kSmallRows = 5 << 19;
-constexpr int64_t kWaitNs = 4000000000LL;
+constexpr long long kWaitNs = 4000000000LL;
+
+// Limit of a launch's barriers; testing: from the environment, so that the
+// blocks give up and the general path takes over (a negative one has run out
+// before the first barrier).
+long long wait_limit(const char *name) {
+  const char *v = getenv(name);
+  return v ? atoll(v) : kWaitNs;
+}
 
 // Blocks of a cooperative launch for about `work` elements: one per SM, fewer
 // for small graphs (two elements per thread).
@@ -549,7 +560,7 @@ int build_small(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, Sup
   TR_TRY(small_grid(rows > n ? rows : n, cfg.sms, &grid));
   SmallArgs a{};
   a.in = in;
-  a.wait_ns = kWaitNs;
+  a.wait_ns = wait_limit("TRUSS_SMALL_BUILD_WAIT_NS");
   a.mask = (unsigned)(slots - 1);
   static_assert(sizeof(SmallCtl) <= ZeroBlock::kCtl && sizeof(OffsetCtl) <= ZeroBlock::kCtl,
                 "control words fit the zero block");
@@ -661,7 +672,7 @@ int small_offsets(Arena &A, const Csr &g, const SupportPrep &prep, const int32_t
   OffsetArgs a{};
   a.n = n;
   a.m = m;
-  a.wait_ns = kWaitNs;
+  a.wait_ns = wait_limit("TRUSS_SMALL_OFFSETS_WAIT_NS");
   a.ctl = (OffsetCtl *)g.zero->offsets;
   a.supA = prep.supA;
   a.supB = prep.supB;

@@ -1136,11 +1136,13 @@ int run_support(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportPrep
   }
   int64_t total = 0;
   int done = TRUSS_ETIMEOUT;  // small graphs: in one launch, unless its blocks cannot meet in time
+  const std::vector<size_t> mk = A.mark();
   if (pre.valid)
     done = small_offsets(A, g, pre, recs ? cuv : nullptr, cfg.sms, sup, toff, &total, &out->small,
                          s);
   if (done != TRUSS_OK) {
     if (done != TRUSS_ETIMEOUT) return done;
+    A.rewind(mk);
     out->small = SmallLists{};
     int64_t *sup64 = A.get<int64_t>(m + 1);
     if (!sup64) return TRUSS_ENOMEM;

@@ -144,3 +144,44 @@ def test_batch_ranked_by_graph_on_the_general_path(general, name):
         ref = oracle.truss(int(n[i]), src[a:b], dst[a:b])
         assert np.array_equal(sup[a:b], ref.support) and np.array_equal(tr[a:b], ref.truss)
         assert kmax[i] == ref.kmax
+
+
+def _give_up_graphs():
+    s, d = graphgen.rmat_raw(13, 60_001, seed=8)
+    yield "rmat", 1 << 13, s, d
+    yield "tiny", *graphgen.tiny()
+
+
+@pytest.mark.parametrize("build,offsets", [("1", None), ("-1", None), (None, "-1"), (None, "1")])
+def test_general_path_when_the_blocks_cannot_meet(ctx, monkeypatch, build, offsets):
+    # limits that run out in the build's launch, or in the one after the walk of
+    # a graph that was built in one launch: the general path takes over there
+    graphs = list(_give_up_graphs())
+    want = {}
+    for name, n, s, d in graphs:
+        ds, dd = torch.from_numpy(s).cuda(), torch.from_numpy(d).cuda()
+        ctx.decompose(n, ds, dd, torch.empty_like(ds), torch.empty_like(ds))
+        want[name] = ctx.stats()["launches"]
+    G = 30
+    ns, off, src, dst = graphgen.batch(G)
+    sb, db = torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()
+    ref = [torch.empty_like(sb), torch.empty_like(sb),
+           torch.empty(G, dtype=torch.int32, device="cuda")]
+    ctx.decompose_batch(ns, off, sb, db, *ref)
+    if build:
+        monkeypatch.setenv("TRUSS_SMALL_BUILD_WAIT_NS", build)
+    if offsets:
+        monkeypatch.setenv("TRUSS_SMALL_OFFSETS_WAIT_NS", offsets)
+    for name, n, s, d in graphs:
+        check(ctx, n, s, d)
+        ds, dd = torch.from_numpy(s).cuda(), torch.from_numpy(d).cuda()
+        ctx.decompose(n, ds, dd, torch.empty_like(ds), torch.empty_like(ds))
+        if offsets != "1":  # two barriers only: the blocks may meet within 16 polls
+            assert ctx.stats()["launches"] > want[name]
+    got = [torch.full_like(x, -7) for x in ref]
+    ctx.decompose_batch(ns, off, sb, db, *got)
+    assert all(torch.equal(a, b) for a, b in zip(got, ref))
+    monkeypatch.undo()
+    for name, n, s, d in graphs:
+        check(ctx, n, s, d)
+        assert ctx.stats()["launches"] <= want[name]
