@@ -176,7 +176,7 @@ def test_general_path_when_the_blocks_cannot_meet(ctx, monkeypatch, build, offse
         check(ctx, n, s, d)
         ds, dd = torch.from_numpy(s).cuda(), torch.from_numpy(d).cuda()
         ctx.decompose(n, ds, dd, torch.empty_like(ds), torch.empty_like(ds))
-        if offsets != "1":  # two barriers only: the blocks may meet within 16 polls
+        if "-1" in (build, offsets):  # within 1 ns, or 16 polls, the blocks may meet
             assert ctx.stats()["launches"] > want[name]
     got = [torch.full_like(x, -7) for x in ref]
     ctx.decompose_batch(ns, off, sb, db, *got)
