@@ -185,3 +185,20 @@ def test_general_path_when_the_blocks_cannot_meet(ctx, monkeypatch, build, offse
     for name, n, s, d in graphs:
         check(ctx, n, s, d)
         assert ctx.stats()["launches"] <= want[name]
+
+
+@pytest.mark.parametrize("name", ["hub", "four hubs in turn", "one edge", "runs of an edge",
+                                  "three edges in turn"])
+def test_rows_that_share_a_counter_or_a_slot(ctx, name):
+    # neighbouring lanes with the same end, or the same edge, and lanes apart
+    k = 5000
+    i = np.arange(k)
+    src, dst = {"hub": (np.zeros(k, int), i), "four hubs in turn": (i % 4, i + 4),
+                "one edge": (np.ones(k, int), np.full(k, 7)),
+                "runs of an edge": (i // 40, i // 40 + 1),
+                "three edges in turn": (i % 3, (i + 1) % 3)}[name]
+    n = 6000
+    es, ed = graphgen.er(300, 2000, seed=1)
+    src, dst = np.concatenate([src, es]), np.concatenate([dst, ed])
+    flip = np.random.default_rng(2).random(len(src)) < 0.5
+    check(ctx, n, np.where(flip, dst, src), np.where(flip, src, dst))
