@@ -187,6 +187,44 @@ def test_general_path_when_the_blocks_cannot_meet(ctx, monkeypatch, build, offse
         assert ctx.stats()["launches"] <= want[name]
 
 
+def both(ctx, general, n, s, d):
+    a, b = run(ctx, n, s, d), run(general, n, s, d)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1]) and a[2] == b[2]
+    return ctx.stats()["launches"], general.stats()["launches"]
+
+
+@pytest.mark.parametrize("length", [383, 384, 385, 511, 512, 513, 1024, 1025])
+def test_long_out_lists(ctx, general, length):
+    # `length` heads, each joined to length + 40 tails and some to one another:
+    # a tail's list holds every head; two such parts, apart in the ids
+    n, parts = 100_000, []
+    for k in range(2):
+        o = k * 4000
+        a = np.repeat(np.arange(length) + o, length + 40)
+        b = np.tile(np.arange(length + 40) + 2000 + o, length)
+        ex, ey = graphgen.er(length, 2000, seed=length + k)
+        parts += [(a, b), (ex + o, ey + o)]
+    perm = graphgen.permutation(n, seed=length, stream=1)
+    src, dst = (perm[np.concatenate(x)].astype(np.int32) for x in zip(*parts))
+    order = np.random.default_rng(length).permutation(len(src))
+    for rows in (np.arange(len(src)), order):  # a tail's edges together, and scattered
+        s, d = torch.from_numpy(src[rows]).cuda(), torch.from_numpy(dst[rows]).cuda()
+        few, many = both(ctx, general, n, s, d)
+        assert few < many  # the launches of support alone: the small path was taken
+
+
+def test_longest_out_list(ctx):
+    # K_2290 fills the rows: its first vertex has the longest list there can be
+    k, n = 2290, 30_000
+    a = torch.triu_indices(k, k, 1, device="cuda").to(torch.int32)
+    s, d = a[0].contiguous(), a[1].contiguous()
+    assert s.numel() <= SMALL_ROWS
+    sup = torch.full_like(s, -7)
+    ctx.support(n, s, d, sup)
+    assert ctx.stats()["launches"] < 10
+    assert bool((sup == k - 2).all())
+
+
 @pytest.mark.parametrize("name", ["hub", "four hubs in turn", "one edge", "runs of an edge",
                                   "three edges in turn"])
 def test_rows_that_share_a_counter_or_a_slot(ctx, name):
