@@ -610,9 +610,21 @@ __global__ void __launch_bounds__(kBlock, 2) k_small_offsets(OffsetArgs a) {
   }
 }
 
-// Rows and vertices up to which the small paths are taken (see the top).
+// Rows and vertices up to which the small paths are taken (see the top).  Above
+// kSmallAnyRows rows, only with at most kSmallPerVertex rows per vertex: where
+// few vertices share the rows the sorts take fewer passes (a key is two vertex
+// ids), and here more atomics meet and more out-lists are long.  Support,
+// general path / here (ms): random rows, 1.05 M over 4,096 vertices (256 rows
+// each) 1.28 / 1.23; 1.5 M over 8,192 (183) 1.61 / 1.64; 2.1 M over 16,384 (128)
+// 1.62 / 1.65, over 8,192 (256) 2.26 / 2.40; 2.6 M over 16,384 (160) 2.07 / 2.52;
+// Chung-Lu of 2.6 M over 16,384 1.59 / 1.93; cliques K_1000 1.02 / 0.84, K_1200
+// 1.35 / 1.22, fifty of K_300 (2.2 M rows) 1.45 / 1.71.  (Rows that repeat few
+// edges are better off here at any density: 1,000 times 2,600 edges of 3,000
+// vertices 0.44 / 0.21; their sizes do not tell them from the dense ones.)
 constexpr int64_t kSmallRows = 5 << 19;
 static_assert((int64_t)kSortCap * kSortCap >= 2 * kSmallRows, "the longest out-list fits");
+constexpr int64_t kSmallAnyRows = 1 << 20;
+constexpr int64_t kSmallPerVertex = 128;
 constexpr long long kWaitNs = 4000000000LL;
 
 // Limit of a launch's barriers; testing: from the environment, so that the
@@ -752,6 +764,7 @@ int build_graph(Arena &A, const RowsIn &in, const SupportCfg &cfg, Csr *out, Sup
   TR_CUDA(cudaMemsetAsync(out->zero, 0, sizeof(ZeroBlock), s));
   // the scans add up tiles of edge costs in 31 bits
   if (cfg.small_paths && in.rows > 0 && in.rows <= kSmallRows && in.n <= kSmallRows &&
+      (in.rows <= kSmallAnyRows || in.rows <= kSmallPerVertex * in.n) &&
       walk_edge_cost(cfg) <= kSmallRows / 2) {
     const std::vector<size_t> mk = A.mark();
     const int rc = build_small(A, in, cfg, out, prep, s);

@@ -61,9 +61,9 @@ def test_small_graph_of_many_duplicates_fits_the_general_paths_workspace():
     # every distinct edge: with the device taken and a workspace sized by the
     # general path (which a wait limit selects) the call still succeeds.
     from paper_1205_6693_gb300 import truss as T
-    n, rows = 3000, 2_600_000
+    n, rows = 30_000, 2_600_000
     gen = torch.Generator(device="cuda").manual_seed(4)
-    s, d = (torch.randint(0, n, (2600,), dtype=torch.int32, generator=gen,
+    s, d = (torch.randint(0, 3000, (2600,), dtype=torch.int32, generator=gen,
                           device="cuda").repeat(rows // 2600) for _ in range(2))
     ref_sup, ref_tr = torch.empty_like(s), torch.empty_like(s)
     sup, tr = torch.empty_like(s), torch.empty_like(s)

@@ -240,3 +240,14 @@ def test_rows_that_share_a_counter_or_a_slot(ctx, name):
     src, dst = np.concatenate([src, es]), np.concatenate([dst, ed])
     flip = np.random.default_rng(2).random(len(src)) < 0.5
     check(ctx, n, np.where(flip, dst, src), np.where(flip, src, dst))
+
+
+@pytest.mark.parametrize("n,rows,small", [
+    (1 << 10, 1 << 20, True), (1 << 10, (1 << 20) + 1, False),
+    (1 << 14, 1 << 21, True), (1 << 14, (1 << 21) + 1, False)])
+def test_densest_rows_taken_and_one_more(ctx, general, n, rows, small):
+    g = torch.Generator(device="cuda").manual_seed(6)
+    s, d = (torch.randint(0, n, (rows,), dtype=torch.int32, generator=g, device="cuda")
+            for _ in range(2))
+    few, many = both(ctx, general, n, s, d)
+    assert few < many if small else few == many
