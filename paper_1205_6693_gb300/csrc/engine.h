@@ -247,11 +247,50 @@ int run_lists(Arena &A, const Csr &g, const SupportCfg &cfg, const SupportOut &s
               uint32_t *tids, TriLists *out, cudaStream_t s);
 
 // ---------------------------------------------------------------- peel ---
+// SMs to use: a sub-round of a small graph is a chain of dependent round trips
+// whatever the grid, and fewer blocks meet sooner.  Up to kWideWork units of
+// work (list entries and 8 per edge, for the scans) at most half the SMs, down to
+// kFewSms, at kSmWork units each.  Measured (ms, SMs: 24 / 38 / 76 / 152), R-MAT
+// of 65 K rows 1.54 / 1.54 / 1.58 / 1.66, 262 K 3.14 / 3.05 / 3.03 / 3.21, 524 K
+// 4.54 / 4.26 / 4.09 / 4.24, 2.1 M 9.76 / 8.29 / 7.00 / 6.92; Chung-Lu of 3 M rows
+// 11.1 / 10.3 / 9.75 / 10.2, 10 M 32.2 / 27.8 / 24.2 / 24.1.  The other half is
+// free for other streams.
+constexpr int kFewSms = 24;
+constexpr int64_t kSmWork = 250000, kWideWork = 80000000;
+inline int peel_sms(int64_t work, int sms) {
+  if (work >= kWideWork || sms <= 2 * kFewSms) return sms;
+  const int64_t want = work / kSmWork > kFewSms ? work / kSmWork : kFewSms;
+  return want < sms / 2 ? (int)want : sms / 2;
+}
+// SMs of a peel that `most` limits (0: not limited) because it shares the device
+// with others: a wide one, which needs them all and outlasts the others, is not
+// limited (16.8 M R-MAT rows taken while twenty requests of 50 K to 300 K rows
+// wait: 95 ms limited, 79 not).
+inline int peel_share(int64_t work, int sms, int most) {
+  return most > 0 && sms > most && work < kWideWork ? most : sms;
+}
+
+// Runs that the server's workers would take from the queued requests, counted
+// up to `most`: small requests that follow one another go together.
+template <class It>
+inline int queued_runs(It r, It end, int64_t batch_rows, int max_batch, int most) {
+  int runs = 0, in_batch = 0;
+  for (; r != end && runs < most; ++r) {
+    if ((*r)->rows > batch_rows) {
+      in_batch = 0;
+      runs++;
+    } else if (in_batch++ % max_batch == 0) {
+      runs++;
+    }
+  }
+  return runs;
+}
+
 struct PeelCfg {
   int block = 512;
   int variant = 0;  // kernel shape (peel.cu: run_peel)
   int sms = 0;
-  int max_sms = 0;  // use at most this many SMs (0 = no limit)
+  int max_sms = 0;  // see peel_share
   long long wait_ns = 4000000000LL;
   // Optional: edges never removed (their triangles still count), and the
   // last level to run (0 = all).  Edges not removed by then get truss 0.

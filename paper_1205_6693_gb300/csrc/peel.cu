@@ -918,23 +918,8 @@ int run_peel(Arena &A, const Csr &g, const SupportOut &so, const TriLists &L, co
   TR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kPeelBlock, 0));
   if (occ < 1) return TRUSS_ECUDA;
   if (variant != 2 && !cfg.count && occ > 1) occ = 1;
-  // SMs to use: a sub-round of a small graph is a chain of dependent round
-  // trips whatever the grid, and fewer blocks meet sooner.  Up to kWideWork
-  // units of work (list entries and 8 per edge, for the scans) at most half
-  // the SMs, down to kFewSms, at kSmWork units each.  Measured (ms, SMs:
-  // 24 / 38 / 76 / 152), R-MAT of 65 K rows 1.54 / 1.54 / 1.58 / 1.66, 262 K
-  // 3.14 / 3.05 / 3.03 / 3.21, 524 K 4.54 / 4.26 / 4.09 / 4.24, 2.1 M 9.76 /
-  // 8.29 / 7.00 / 6.92; Chung-Lu of 3 M rows 11.1 / 10.3 / 9.75 / 10.2, 10 M
-  // 32.2 / 27.8 / 24.2 / 24.1.  The other half is free for other streams.
-  constexpr int kFewSms = 24;
-  constexpr int64_t kSmWork = 250000, kWideWork = 80000000;
-  const int64_t work = so.entries + 8 * m;
-  if (variant == 2 && work < kWideWork) {
-    const int64_t want = work / kSmWork > kFewSms ? work / kSmWork : kFewSms;
-    if (sms > 2 * kFewSms && want < sms / 2) sms = (int)want;
-    else if (sms > 2 * kFewSms) sms = sms / 2;
-  }
-  if (cfg.max_sms > 0 && sms > cfg.max_sms) sms = cfg.max_sms;
+  if (variant == 2) sms = peel_sms(so.entries + 8 * m, sms);
+  sms = peel_share(so.entries + 8 * m, sms, cfg.max_sms);
   PeelArgs a{};
   a.m = m;
   a.sup = so.sup;

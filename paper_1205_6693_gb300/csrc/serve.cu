@@ -188,6 +188,15 @@ bool fits(const truss_server *S, const Request *r, int extra_count, int64_t extr
   return S->inflight_fp + extra_fp + r->fp <= S->o.hbm_budget_bytes;
 }
 
+// Runs that idle workers would take from the queue as it stands.
+int runs_next(const truss_server *S) {
+  auto end = S->pending.begin();
+  int64_t fp = 0;
+  for (int count = 0; end != S->pending.end() && fits(S, *end, count, fp); ++end, count++)
+    fp += (*end)->fp;
+  return tr::queued_runs(S->pending.begin(), end, S->o.batch_rows, S->o.max_batch, S->o.streams);
+}
+
 void worker_main(truss_server *S) {
   truss_ctx *ctx = nullptr;
   cudaStream_t st = nullptr;
@@ -224,12 +233,13 @@ void worker_main(truss_server *S) {
       S->admitted += (int64_t)job.size();
       S->launches++;
       S->busy++;
-      sharers = (int)std::min<int64_t>(S->o.streams, S->busy + (int64_t)S->pending.size());
+      sharers = std::min(S->o.streams, S->busy + runs_next(S));
     }
     if (rc == TRUSS_OK) {
       // The peel is a chain of short phases that leaves most of its SMs idle,
       // so runs that overlap take a share each instead of one after another
-      // (24 requests of 1 K to 2 M rows: 20.2 -> 19.0 ms).
+      // (24 requests of 1 K to 2 M rows: 20.2 -> 19.0 ms).  The waiting requests
+      // count as the runs they will make: twenty tiny ones are one.
       tr::ctx_set_peel_sms(ctx, sharers > 1 ? tr::ctx_sms(ctx) / sharers : 0);
       // workspace cap of this run: twice the projection, or the whole budget
       // for a request queued again after running out of its cap
