@@ -106,11 +106,12 @@ __global__ void k_vertex_base(int64_t n, int G, const int64_t *voff, int32_t *vb
 // Sort key of each vertex: its degree, behind its graph's number in a batch
 // (recovered from the order of the first vertices: vertices are numbered graph
 // by graph, so the stable sort only needs graphs to differ).
-__global__ void k_degree_keys(int64_t n, int db, int G, const int64_t *voff, const int32_t *deg,
-                              uint32_t *key, int32_t *id) {
+// The keys take the place of the degrees.
+__global__ void k_degree_keys(int64_t n, int db, int G, const int64_t *voff, uint32_t *deg,
+                              int32_t *id) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    key[v] = (uint32_t)deg[v] | (uint32_t)(db < 32 ? graph_of_row(voff, G, v) : 0) << (db & 31);
+    if (db < 32) deg[v] |= (uint32_t)graph_of_row(voff, G, v) << db;
     id[v] = (int32_t)v;
   }
 }
@@ -141,14 +142,13 @@ __global__ void k_iota(int64_t n, int32_t *x) {
     x[i] = (int32_t)i;
 }
 
-// Ranks of the sorted vertices, and their degrees (the low db bits of the key).
-__global__ void k_newid(int64_t n, int db, const uint32_t *skey, const int32_t *order,
-                        int32_t *newid, int32_t *sdeg) {
-  const uint32_t mask = db < 32 ? (1u << db) - 1u : 0xFFFFFFFFu;
+// Ranks of the sorted vertices, and their degrees (the low db bits of the
+// sorted keys) in the place of the keys.
+__global__ void k_newid(int64_t n, int db, const int32_t *order, int32_t *newid, uint32_t *skey) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     newid[order[i]] = (int32_t)i;
-    sdeg[i] = (int32_t)(skey[i] & mask);
+    if (db < 32) skey[i] &= (1u << db) - 1u;
   }
 }
 
@@ -282,9 +282,8 @@ int build_csr(Arena &A, const RowsIn &in, Csr *out, int32_t *d_err, cudaStream_t
 
   // 3. degrees and rank
   int32_t *deg = A.get<int32_t>(n), *sdeg = A.get<int32_t>(n);
-  uint32_t *dkey = A.get<uint32_t>(n), *skey = A.get<uint32_t>(n);
   int32_t *ids = A.get<int32_t>(n), *order = A.get<int32_t>(n), *newid = A.get<int32_t>(n);
-  if (!deg || !sdeg || !dkey || !skey || !ids || !order || !newid) return TRUSS_ENOMEM;
+  if (!deg || !sdeg || !ids || !order || !newid) return TRUSS_ENOMEM;
   TR_CUDA(cudaMemsetAsync(deg, 0, sizeof(int32_t) * n, s));
   if (m > 0) {
     k_degree<<<grid_for(m, kBlock, maxg), kBlock, 0, s>>>(m, U, V, deg);
@@ -294,8 +293,8 @@ int build_csr(Arena &A, const RowsIn &in, Csr *out, int32_t *d_err, cudaStream_t
   const int db = local ? nb : 32;
   const int mb = bits_for((uint64_t)(m > 0 ? m : 1));
   const int dbits = local ? nb + gb : (b < mb ? b : mb);
-  k_degree_keys<<<grid_for(n, kBlock, maxg), kBlock, 0, s>>>(n, db, in.graphs, in.voff, deg, dkey,
-                                                             ids);
+  uint32_t *dkey = (uint32_t *)deg, *skey = (uint32_t *)sdeg;
+  k_degree_keys<<<grid_for(n, kBlock, maxg), kBlock, 0, s>>>(n, db, in.graphs, in.voff, dkey, ids);
   TR_LAUNCHED();
   tb = 0;
   TR_TRY(sort_pairs_u32(nullptr, &tb, dkey, skey, ids, order, n, 0, dbits, s));
@@ -304,7 +303,7 @@ int build_csr(Arena &A, const RowsIn &in, Csr *out, int32_t *d_err, cudaStream_t
   TR_TRY(sort_pairs_u32(tmp, &tb, dkey, skey, ids, order, n, 0, dbits, s));
   out->order = order;
   out->sdeg = sdeg;
-  k_newid<<<grid_for(n, kBlock, maxg), kBlock, 0, s>>>(n, db, skey, order, newid, sdeg);
+  k_newid<<<grid_for(n, kBlock, maxg), kBlock, 0, s>>>(n, db, order, newid, skey);
   TR_LAUNCHED();
 
   // 4. orientation

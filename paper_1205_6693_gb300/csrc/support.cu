@@ -1020,27 +1020,25 @@ int prepare_walk(Arena &A, const Csr &g, const SupportCfg &cfg, SupportPrep *out
   int32_t *supA = A.get<int32_t>(m), *supB = A.get<int32_t>(m);
   int64_t *wcost = A.get<int64_t>(m + 1), *wpre = A.get<int64_t>(m + 1);
   int64_t *wbound = A.get<int64_t>(m + 1), *tbpre = A.get<int64_t>(m + 1);
-  int64_t *hcnt = A.get<int64_t>(n + 1);
   int64_t *inoff = A.get<int64_t>(n + 1);
   int32_t *inedge = A.get<int32_t>(m), *ihead = A.get<int32_t>(m);
-  if (!supA || !supB || !wcost || !wpre || !wbound || !tbpre || !hcnt || !inoff || !inedge ||
-      !ihead)
+  if (!supA || !supB || !wcost || !wpre || !wbound || !tbpre || !inoff || !inedge || !ihead)
     return TRUSS_ENOMEM;
   TR_CUDA(cudaMemsetAsync(supA, 0, sizeof(int32_t) * m, s));
   TR_CUDA(cudaMemsetAsync(supB, 0, sizeof(int32_t) * m, s));
   int64_t W = 0, R = 0;
   if (m > 0) {
-    // edges grouped by head: in-degrees and their prefix give each head's
-    // group; a stable radix sort of (head, edge id) fills the groups in
+    // edges grouped by head: the prefix of the in-degrees (scanned in place)
+    // gives each head's group; a stable radix sort of (head, edge id) fills the groups in
     // edge order (the edge ids sit in wcost's memory until the sort)
-    k_in_degree<<<grid_for(n + 1, 256, 152 * 16), 256, 0, s>>>(n, g.sdeg, g.offp, hcnt);
+    k_in_degree<<<grid_for(n + 1, 256, 152 * 16), 256, 0, s>>>(n, g.sdeg, g.offp, inoff);
     TR_LAUNCHED();
     int32_t *ids = (int32_t *)wcost;
     k_seq<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(m, ids);
     TR_LAUNCHED();
     const int hbits = bits_for((uint64_t)(n > 1 ? n - 1 : 1));
     size_t tb = 0, tb2 = 0, tb3 = 0;
-    TR_TRY(exclusive_sum_i64(nullptr, &tb, hcnt, inoff, n + 1, s));
+    TR_TRY(exclusive_sum_i64(nullptr, &tb, inoff, inoff, n + 1, s));
     TR_TRY(exclusive_sum_i64(nullptr, &tb2, wcost, wpre, m + 1, s));
     TR_TRY(sort_pairs_u32(nullptr, &tb3, (const uint32_t *)g.adjp, (uint32_t *)ihead, ids, inedge,
                           m, 0, hbits, s));
@@ -1048,7 +1046,7 @@ int prepare_walk(Arena &A, const Csr &g, const SupportCfg &cfg, SupportPrep *out
     tb2 = tb2 > tb3 ? tb2 : tb3;
     void *tmp = A.alloc(tb2);
     if (!tmp) return TRUSS_ENOMEM;
-    TR_TRY(exclusive_sum_i64(tmp, &tb, hcnt, inoff, n + 1, s));
+    TR_TRY(exclusive_sum_i64(tmp, &tb, inoff, inoff, n + 1, s));
     TR_TRY(sort_pairs_u32(tmp, &tb3, (const uint32_t *)g.adjp, (uint32_t *)ihead, ids, inedge, m,
                           0, hbits, s));
     const int ec = walk_edge_cost(cfg);

@@ -86,3 +86,25 @@ def test_small_graph_of_many_duplicates_fits_the_general_paths_workspace():
         hold.clear()
         ctx.close()
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("graphs", [1, 100])
+def test_workspace_per_vertex_of_the_general_path(graphs):
+    # what a vertex adds where vertices outnumber rows: fifteen words, before its
+    # degree was sorted with its graph's number
+    from paper_1205_6693_gb300 import truss as T
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    peaks = []
+    for n in (4_000_000, 8_000_000):  # above the one-launch build's limit
+        s, d = (torch.randint(0, n // graphs, (60_000,), dtype=torch.int32, generator=gen,
+                              device="cuda") for _ in range(2))
+        sup, tr = torch.empty_like(s), torch.empty_like(s)
+        ctx = T.Context(0)
+        if graphs == 1:
+            ctx.decompose(n, s, d, sup, tr)
+        else:
+            off = np.arange(graphs + 1, dtype=np.int64) * (60_000 // graphs)
+            ctx.decompose_batch(np.full(graphs, n // graphs, np.int64), off, s, d, sup, tr)
+        peaks.append(ctx.stats()["workspace_peak"])
+        ctx.close()
+    assert (peaks[1] - peaks[0]) / 4_000_000 <= 60.2
