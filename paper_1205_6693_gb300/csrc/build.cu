@@ -207,10 +207,13 @@ int build_csr(Arena &A, const RowsIn &in, Csr *out, int32_t *d_err, cudaStream_t
   out->rows = rows;
   const int b = bits_for(n > 1 ? (uint64_t)(n - 1) : 1);
   // a batch whose graph numbers and degrees fit 32 bits together is ranked
-  // graph by graph, with heads local to their graph
+  // graph by graph, with heads local to their graph, unless its vertices
+  // outnumber its rows: each is looked up in its graph twice (1,000 graphs of
+  // 5,000 vertices and 100 rows: 0.83 ms so, 0.75 mixed; of 4,000 vertices and
+  // 3,000 rows 1.68 / 1.66)
   const int gb = bits_for((uint64_t)(in.graphs > 1 ? in.graphs - 1 : 0));
   const int nb = bits_for(in.max_n > 1 ? (uint64_t)(in.max_n - 1) : 1);
-  const bool local = in.graphs > 1 && in.max_n > 0 && gb + nb < 32;
+  const bool local = in.graphs > 1 && in.max_n > 0 && n <= rows && gb + nb < 32;
   const int lb = local ? nb : b, kbits = b + lb;
   const uint64_t sentinel = kbits >= 64 ? ~0ull : ((1ull << kbits) - 1);
 

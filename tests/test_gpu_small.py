@@ -251,3 +251,22 @@ def test_densest_rows_taken_and_one_more(ctx, general, n, rows, small):
             for _ in range(2))
     few, many = both(ctx, general, n, s, d)
     assert few < many if small else few == many
+
+
+@pytest.mark.parametrize("spare", [0, 1])
+def test_batch_of_as_many_vertices_as_rows(general, spare):
+    # ranked graph by graph up to there, in one order with a vertex more
+    G, rows = 60, 200
+    n = np.full(G, rows, np.int64)
+    n[-1] += spare
+    off = np.arange(G + 1, dtype=np.int64) * rows
+    rng = np.random.default_rng(spare)
+    src, dst = (rng.integers(0, 40, G * rows).astype(np.int32) for _ in range(2))
+    s, d = torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()
+    sup, tr = torch.full_like(s, -7), torch.full_like(s, -7)
+    general.decompose_batch(n, off, s, d, sup, tr)
+    sup, tr = sup.cpu().numpy(), tr.cpu().numpy()
+    for i in range(G):
+        a, b = off[i], off[i + 1]
+        ref = oracle.truss(int(n[i]), src[a:b], dst[a:b])
+        assert np.array_equal(sup[a:b], ref.support) and np.array_equal(tr[a:b], ref.truss)
