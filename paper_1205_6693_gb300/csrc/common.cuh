@@ -239,13 +239,14 @@ __device__ __forceinline__ uint32_t reserve_items(unsigned long long *w, int n) 
   return (uint32_t)(atomicAdd(w, (unsigned long long)(unsigned)n << kItemShift) >> kItemShift);
 }
 
-// End of a phase: a barrier of the whole grid, after which *items is the number of items the phase appended and, for a
-// scan, *so is what it found.  The count shares its word with the barrier's
+// End of a phase: a barrier of the whole grid, after which *items is the number
+// of items the phase appended and, for a scan, *so is what it found.  The count
+// shares its word with the barrier's
 // arrivals, so the load that sees the last arrival brings it along, and one
 // thread per block reads and passes it on: read by every warp, one L2 sector
 // served 4,864 requests per value and barrier (edge peel: 1.1 us of each
-// sub-round, 5 to 7 us of each scan).  A grid barrier that waits longer than wait_ns
-// records TRUSS_ETIMEOUT.  Returns false if some block has recorded an error.
+// sub-round, 5 to 7 us of each scan).  A grid barrier that waits longer than
+// wait_ns records TRUSS_ETIMEOUT.  Returns false if some block has recorded an error.
 __device__ __forceinline__ bool phase_end(PhaseCtl *ctl, long long wait_ns, unsigned ph,
                                           uint32_t *items, const ScanOut *scan, ScanOut *so) {
   __shared__ unsigned long long s_word2[2];  // by phase parity: read until the next phase ends

@@ -34,7 +34,7 @@ constexpr int kMaxRows = TRUSS_NOALLOC_MAX_ROWS;
 constexpr int kMaxN = TRUSS_NOALLOC_MAX_N;
 constexpr int kSlots = 4 * kMaxRows;  // hash slots (load <= 1/4)
 constexpr int kThreads = 256;
-constexpr int kGroup = 16;  // lanes that walk one edge's shorter list
+constexpr int kGroup = 16;  // lanes that walk the out-list of one edge's lower end
 constexpr unsigned long long kEmpty = ~0ull;
 
 // Layout of the scratch array (element counts).

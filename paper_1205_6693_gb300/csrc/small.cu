@@ -17,11 +17,12 @@
 // What bounds it: a few dependent L2 round trips (540 clocks each) and a grid
 // barrier (1.3 us) per phase, then the hash table's and the cursors' atomics.
 //
-// Build, support and lists, general path / here (ms): the 4,096-vertex graph
-// 0.43 / 0.18, R-MAT of 65 K rows 0.46 / 0.22, 524 K 1.04 / 0.79, 2.1 M 2.52 /
-// 2.39, 4.2 M 4.83 / 4.95; Chung-Lu of 200 K rows 0.62 / 0.31, 1 M 1.32 / 1.08,
-// 2 M 1.80 / 1.71, 4 M 3.00 / 3.41.  Above kSmallRows rows the table and the
-// lists leave L2, and the sorts, which stream, are faster.
+// Decompose, general path / here (ms): 1.5 M R-MAT rows over 262,144 vertices
+// 5.87 / 5.60, 2.1 M 7.97 / 7.71, 2.6 M 9.54 / 9.59; 2.6 M Chung-Lu rows over
+// 1,048,576 vertices 8.19 / 8.42, random rows 1.40 / 1.28.  Support alone: 65 K
+// R-MAT rows over 16,384 vertices 0.46 / 0.17, 262 K 0.53 / 0.27, 1.05 M 0.98 /
+// 0.86.  Above kSmallRows rows the table and the lists leave L2, and the sorts,
+// which stream, are faster.
 #include <climits>
 #include <cstdlib>
 
